@@ -14,6 +14,7 @@
 
 #include "dgpe.h"
 #include "dgpe_kernels.cuh"
+#include "dgpe_lines.h"
 
 namespace dgpe {
 
@@ -232,6 +233,11 @@ template <typename R> struct EngineT : Engine {
   double tau[3] = {0, 0, 0};
   // chunk-scan reach of the FP32 chunk-parallel CN solve per axis (cn_line_st)
   int cn_dlim[3] = {0, 0, 0};
+  // constant-coefficient CN form of each axis (FP32 bulk; dl = 0: tables):
+  // imaginary time, real time, and real time conjugated for the reverse step
+  CnConst<float> cn_kr[3] = {};
+  CnConst<float2> cn_kc[3] = {}, cn_ka[3] = {};
+  int cols_pgrid[3] = {0, 0, 0};  // persistent grid of the strided CN passes (dgpe_cols.cu)
 
   // pass configurations
   int x_LP = 0, x_T = 0, x_TPL = 0, x_C = 0, x_pitchz = 0, x_pitch = 0, x_grid = 0;
@@ -465,6 +471,7 @@ template <typename R> struct EngineT : Engine {
     if ((rc = dalloc(&dip_part, (size_t)std::max(ndip, 1)))) return rc;
     if ((rc = dalloc(&obs_out, OBS_COUNT + 1))) return rc;
     if ((rc = set_smem_attrs())) return rc;
+    setup_lines();
     DGPE_CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
     use_graph = !(p.flags & DGPE_FLAG_NO_GRAPH);
     strang = (p.flags & DGPE_FLAG_STRANG) != 0;
@@ -560,6 +567,31 @@ template <typename R> struct EngineT : Engine {
     return upload(U, hu);
   }
 
+  // Constant-coefficient form of the CN solve with kt (dgpe_lines.cuh), FP64
+  // then rounded.  dl chunks reach to below 2^-32 (of the largest chunk
+  // value: |alpha|^(CL dl) / (1 - |alpha|^CL)); beyond CN_DL chunks, or where
+  // that is the whole line, the tables are used (dl = 0).  J: the sites of a
+  // chunk an inflow changes by more than 2^-32 of it.
+  template <typename Coef> static CnConst<Coef> cn_const(zd kt, int cl, int tpl) {
+    const zd m = 2.0 / (1.0 + 2.0 * kt + std::sqrt(1.0 + 4.0 * kt)), al = kt * m, pc = std::pow(al, cl);
+    auto put = [](Coef &c, zd v) {
+      if constexpr (std::is_same<Coef, float2>::value) { c.x = (float)v.real(); c.y = (float)v.imag(); }
+      else c = (float)v.real();
+    };
+    CnConst<Coef> K{};
+    put(K.al, al);
+    put(K.m2, -2.0 * kt * m);
+    put(K.pc, pc);
+    zd p = 1.0;
+    for (int i = 0; i < CN_PW; ++i) { p *= al; put(K.pw[i], p); }
+    const double rho = std::abs(pc), lim = 0x1p-32 * (1.0 - rho);
+    for (int dl = 1; dl <= std::min<int>(CN_DL, tpl); ++dl)
+      if (std::pow(rho, dl) <= lim) { K.dl = dl; break; }
+    K.J = 1;
+    while (K.J < cl && std::pow(std::abs(al), K.J + 1) > 0x1p-32) ++K.J;
+    return K;
+  }
+
   // Crank-Nicolson LU and chunk-scan tables for axis a: m, alpha, P, Q (n
   // each), then the middle-row pivot mu of the two-ended elimination.
   int build_cn_tables() {
@@ -599,6 +631,9 @@ template <typename R> struct EngineT : Engine {
         if (dl >= 64) dl = 0;
       }
       cn_dlim[a] = dl;
+      cn_kr[a] = cn_const<float>(zd(tau[a], 0.0), C, n / C);
+      cn_kc[a] = cn_const<float2>(zd(0.0, tau[a]), C, n / C);
+      cn_ka[a] = cn_const<float2>(zd(0.0, -tau[a]), C, n / C);
       if (!cntab[a]) {
         int rc = dalloc((Cx **)&cntab[a], 4 * (size_t)n + 1);
         if (rc) return rc;
@@ -739,36 +774,15 @@ template <typename R> struct EngineT : Engine {
         return DGPE_OK;
       });
       if (rc) return rc;
+      if constexpr (sizeof(R) == 4) continue;  // FP32: dgpe_cols.cu
       rc = with_cl(var[a], [&](auto CLc) -> int {
         constexpr int CL = decltype(CLc)::value;
         int r;
-        const size_t one = cn[a].smem, two = 2 * cn[a].smem;
-        if ((r = smem_attr(k_cn_strided<R, R, CL>, one))) return r;
-        if ((r = smem_attr(k_cn_strided<R, Cx, CL>, one))) return r;
+        const size_t two = 2 * cn[a].smem;
         if ((r = smem_attr(k_cn_strided_pipe<R, R, CL>, two))) return r;
         if ((r = smem_attr(k_cn_strided_pipe<R, Cx, CL>, two))) return r;
         if ((r = smem_attr(k_cn_strided_pipe<R, R, CL, false>, two))) return r;
         if ((r = smem_attr(k_cn_strided_pipe<R, Cx, CL, false>, two))) return r;
-        if constexpr (sizeof(R) == 4 && CL == 16) {
-          r = with_pow2_len(cn[a].n, [&](auto Nc) -> int {
-            constexpr int N = decltype(Nc)::value;
-            if constexpr (N != 0) {
-              int q;
-              if constexpr (16 * (N / 16) <= DGPE_MAXT) {
-                if ((q = smem_attr(k_cn_pipe_ct<R, R, 16, true, N, 16>, two))) return q;
-                if ((q = smem_attr(k_cn_pipe_ct<R, R, 16, false, N, 16>, two))) return q;
-                if ((q = smem_attr(k_cn_pipe_ct<R, Cx, 16, false, N, 16>, two))) return q;
-              }
-              if constexpr (8 * (N / 16) <= DGPE_MAXT) {
-                if ((q = smem_attr(k_cn_pipe_ct<R, R, 16, true, N, 8>, two))) return q;
-                if ((q = smem_attr(k_cn_pipe_ct<R, R, 16, false, N, 8>, two))) return q;
-                if ((q = smem_attr(k_cn_pipe_ct<R, Cx, 16, false, N, 8>, two))) return q;
-              }
-            }
-            return DGPE_OK;
-          });
-          if (r) return r;
-        }
         // persistent grid: as many CTAs as fit on the device, at most one per
         // tile, each double-buffered (the next tile is prefetched)
         const int ntiles = (int)(cn[a].grid.x * cn[a].grid.y);
@@ -782,6 +796,15 @@ template <typename R> struct EngineT : Engine {
       if (rc) return rc;
     }
     return setup_tma();
+  }
+
+  // Persistent grids of the register-resident line passes for the current mode.
+  void setup_lines() {
+    if constexpr (sizeof(R) == 4) {
+      for (int a = 1; a < dim; ++a)
+        cols_pgrid[a] = cols_grid(cn[a].n, cn[a].C, (unsigned)cn[a].ncols * cn[a].grid.y, nsm, imag != 0,
+                                  (imag ? cn_kr[a].dl : cn_kc[a].dl) == 0);
+    }
   }
 
   // ------------------------------------------------------------- launches
@@ -970,36 +993,27 @@ template <typename R> struct EngineT : Engine {
     DGPE_LCK(__func__);
     return DGPE_OK;
   }
-  // FP32, power-of-two length, tile width 16 or 8: the length-specialised
-  // CN pass (same grid, block and shared memory as k_cn_strided_pipe)
-  bool launch_cn_ct(const CnCfg &c, int axis, const CArgs<R> &A, int ncb, int ntiles, cudaStream_t s) {
-    if constexpr (sizeof(R) != 4) {
-      return false;
-    } else {
-      if (var[axis] != VAR_P2 || !(c.W == 16 || c.W == 8)) return false;
-      return with_pow2_len(c.n, [&](auto Nc) -> int {
-        constexpr int N = decltype(Nc)::value;
-        if constexpr (N == 0) {
-          return 0;
-        } else {
-          auto go = [&](auto Wc) {
-            constexpr int WW = decltype(Wc)::value;
-            if constexpr (WW * (N / 16) <= DGPE_MAXT) {
-              if (imag && A.norm) k_cn_pipe_ct<R, R, 16, true, N, WW><<<c.pgrid[0], c.T, 2 * c.smem, s>>>(A, ncb, ntiles);
-              else if (imag) k_cn_pipe_ct<R, R, 16, false, N, WW><<<c.pgrid[0], c.T, 2 * c.smem, s>>>(A, ncb, ntiles);
-              else k_cn_pipe_ct<R, Cx, 16, false, N, WW><<<c.pgrid[1], c.T, 2 * c.smem, s>>>(A, ncb, ntiles);
-              return 1;
-            } else {
-              return 0;
-            }
-          };
-          return (c.W == 16) ? go(std::integral_constant<int, 16>{}) : go(std::integral_constant<int, 8>{});
-        }
-      }) != 0;
+  // FP32: the register-resident strided solve
+  int launch_cols(int axis, bool final_pass, cudaStream_t s, Cx *buf, bool adjoint) {
+    if constexpr (sizeof(R) == 4) {
+      const CnCfg &c = cn[axis];
+      ColArgs A{};
+      A.psi = buf ? buf : psi;
+      A.cntab = adjoint ? cntab_adj[axis] : cntab[axis];
+      A.prm = prm; A.partial = partial; A.counter = counter; A.step = dstep;
+      A.es = c.es; A.os = c.os; A.ncols = (unsigned)c.ncols; A.tot = (unsigned)c.ncols * c.grid.y;
+      A.n = c.n; A.cl = c.C; A.final_pass = final_pass ? 1 : 0; A.norm = (final_pass && imag) ? 1 : 0;
+      A.dlim = cn_dlim[axis]; A.tau = adjoint ? -tau[axis] : tau[axis];
+      const cudaError_t e = imag ? cols_launch(A, cn_kr[axis], cols_pgrid[axis], s)
+                                 : cols_launch(A, adjoint ? cn_ka[axis] : cn_kc[axis], cols_pgrid[axis], s);
+      launched(1);
+      if (e != cudaSuccess) { err = std::string("launch of the CN pass: ") + cudaGetErrorString(e); return DGPE_ECUDA; }
     }
+    return DGPE_OK;
   }
   int launch_cn(int axis, bool final_pass, cudaStream_t s, Cx *buf = nullptr, bool adjoint = false) {
     if (cn_serial) return launch_lines(axis, final_pass, s, buf, adjoint);
+    if constexpr (sizeof(R) == 4) return launch_cols(axis, final_pass, s, buf, adjoint);
     const CnCfg &c = cn[axis];
     CArgs<R> A{};
     A.psi = buf ? buf : psi; A.cntab = adjoint ? cntab_adj[axis] : cntab[axis];
@@ -1009,11 +1023,6 @@ template <typename R> struct EngineT : Engine {
     A.norm = (final_pass && imag) ? 1 : 0; A.tau = adjoint ? -tau[axis] : tau[axis];
     A.cnd = cn_dlim[axis];
     const int ncb = (int)c.grid.x, ntiles = (int)(c.grid.x * c.grid.y);
-    if (launch_cn_ct(c, axis, A, ncb, ntiles, s)) {
-      launched(1);
-      DGPE_LCK(__func__);
-      return DGPE_OK;
-    }
     with_cl(var[axis], [&](auto CLc) -> int {
       constexpr int CL = decltype(CLc)::value;
       // the norm's code only in the pass that takes the norm
@@ -1490,6 +1499,7 @@ template <typename R> struct EngineT : Engine {
     p.mode = mode;
     imag = (mode == DGPE_IMAG);
     if ((rc = build_cn_tables())) return rc;
+    setup_lines();
     if (use_graph && (rc = capture())) return rc;
     return DGPE_OK;
   }

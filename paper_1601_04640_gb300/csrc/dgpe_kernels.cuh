@@ -1121,10 +1121,6 @@ __device__ __forceinline__ void cn_strided_body(const CArgs<R> &A, int bx, int b
   }
 }
 template <typename R, typename Coef, int CL, bool NORM = true>
-__global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB(R)) k_cn_strided(const __grid_constant__ CArgs<R> A) {
-  cn_strided_body<R, Coef, CL, NORM>(A, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
-}
-template <typename R, typename Coef, int CL, bool NORM = true>
 __global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB(R)) k_cn_strided_batch(const CArgs<R> *__restrict__ args) {
   __shared__ CArgs<R> sA;
   const CArgs<R> &A = block_args(args, sA);
@@ -1188,99 +1184,6 @@ __global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB_CN(R)) k_cn_strided_pipe(
 #pragma unroll
       for (int i = 0; i < CL; ++i) {
         const int a = r0 + i * A.TPL;
-        const cx<R> v = tb[lc * P + a + a / CL];
-        dst[(size_t)a * es] = v;
-        if (NORM && A.norm) ts += v.x * v.x + v.y * v.y;
-      }
-      if (NORM && A.norm) acc += (double)ts;
-    }
-    __syncthreads();  // the buffer is refilled two iterations later
-  }
-  cp_async_wait<0>();
-  if (!A.final_pass) return;
-  const unsigned nblk = gridDim.x;
-  if (NORM && A.norm) {
-    double sblk = block_sum(acc, red);
-    if (threadIdx.x == 0) A.partial[blockIdx.x] = sblk;
-  }
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned ticket = atomicAdd(A.counter, 1u);
-    am_last = (ticket == nblk - 1);
-  }
-  __syncthreads();
-  if (!am_last) return;
-  __threadfence();
-  if (NORM && A.norm) {
-    double sum = 0.0;
-    for (unsigned i = threadIdx.x; i < nblk; i += blockDim.x) sum += __ldcg(A.partial + i);
-    sum = block_sum(sum, red);
-    if (threadIdx.x == 0) {
-      const double norm = A.prm[PRM_CELL] * sum;
-      if (norm > 0.0 && isfinite(norm)) A.prm[PRM_SC] = 1.0 / sqrt(norm);
-      else A.prm[PRM_NONFINITE] = 1.0;
-    }
-  }
-  if (threadIdx.x == 0) {
-    *A.step += 1;
-    *A.counter = 0u;
-  }
-}
-
-// The same pass with the line length N and tile width W as compile-time
-// constants (FP32, power-of-two lengths): every index folds.
-template <typename R, typename Coef, int CL, bool NORM, int N, int W>
-__global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB_CN(R)) k_cn_pipe_ct(const __grid_constant__ CArgs<R> A, int ncb, int ntiles) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ double red[32];
-  __shared__ int am_last;
-  constexpr int n = N, TPL = N / CL, P = N + N / CL + 1, lW = ct_log2(W);
-  static_assert(W * TPL <= DGPE_MAXT, "block size");
-  cx<R> *const buf0 = reinterpret_cast<cx<R> *>(smraw);  // buffer k at buf0 + k W P
-  const long long es = A.estride;
-  const int lc = threadIdx.x & (W - 1), r0 = threadIdx.x >> lW;
-  auto fetch = [&](int tile, cx<R> *tb) {
-    const int cb = tile % ncb, o = tile / ncb;
-    const int c0 = cb * W;
-    if (c0 + lc < A.ncols) {
-      const cx<R> *src = A.psi + (size_t)o * A.ostride + c0 + lc;
-#pragma unroll
-      for (int i = 0; i < CL; ++i) {
-        const int a = r0 + i * TPL;
-        cp_async_elem(tb + lc * P + a + a / CL, src + (size_t)a * es);
-      }
-    }
-    cp_async_commit();
-  };
-  constexpr bool TAB = (sizeof(R) == 8);
-  __shared__ __align__(16) Coef s_tab[TAB ? 1 : 4 * P];
-  if (!TAB) stage_cn_tables<Coef, CL>(s_tab, reinterpret_cast<const Coef *>(A.cntab), n);  // visible after the loop's first barrier
-  double acc = 0.0;
-  int k = 0;
-  if ((int)blockIdx.x < ntiles) fetch(blockIdx.x, buf0);
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, k ^= 1) {
-    const int next = tile + gridDim.x;
-    if (next < ntiles) fetch(next, buf0 + (k ^ 1) * W * P);
-    else cp_async_commit();  // keep one group per iteration
-    cp_async_wait<1>();      // this tile's copies are done (the next may be in flight)
-    __syncthreads();
-    const int cb = tile % ncb, o = tile / ncb;
-    const int c0 = cb * W;
-    cx<R> *tb = buf0 + k * W * P;
-    const int l = threadIdx.x / TPL, q = threadIdx.x - l * TPL;
-    if constexpr (TAB) cn_line<R, Coef, CL>(tb + l * P, n, TPL, q, make_kt<Coef>(A.tau),
-                                        reinterpret_cast<const Coef *>(A.cntab), c0 + l < A.ncols);
-    else cn_line_st<R, Coef, CL>(tb + l * P, n, TPL, q, make_kt<Coef>(A.tau), s_tab, c0 + l < A.ncols, A.cnd);
-    __syncthreads();
-    if (c0 + lc < A.ncols) {
-      cx<R> *dst = A.psi + (size_t)o * A.ostride + c0 + lc;
-      // |x|^2 of the thread's CL sites summed in R (FP32: an FP64 sum per
-      // site held the FP32 final pass at the FP64 pipe's rate, 0.21 against
-      // 0.08 ms at 256^3), then accumulated in FP64 across tiles and blocks
-      R ts = (R)0;
-#pragma unroll
-      for (int i = 0; i < CL; ++i) {
-        const int a = r0 + i * TPL;
         const cx<R> v = tb[lc * P + a + a / CL];
         dst[(size_t)a * es] = v;
         if (NORM && A.norm) ts += v.x * v.x + v.y * v.y;
