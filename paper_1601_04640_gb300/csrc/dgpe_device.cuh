@@ -183,13 +183,40 @@ template <bool INV, typename C> __device__ __forceinline__ void dft5(C *v) {
   v[1] = a1 + b1; v[4] = a1 - b1;
   v[2] = a2 + b2; v[3] = a2 - b2;
 }
+template <int RAD, bool INV, typename C> __device__ __forceinline__ void dft_small(C *v) {
+  if constexpr (RAD == 3) dft3<INV>(v);
+  else if constexpr (RAD == 4) dft4<INV>(v);
+  else dft5<INV>(v);
+}
+// 12 = 3 x 4 and 20 = 4 x 5 points by Good's prime-factor map: inputs n =
+// (B n1 + A n2) mod AB, outputs k = k1 (mod A) = k2 (mod B); no twiddles.
+template <int A, int B, int EA, int EB, bool INV, typename C> __device__ __forceinline__ void dft_pf(C *v) {
+  C t[B][A];
+#pragma unroll
+  for (int n2 = 0; n2 < B; ++n2) {
+#pragma unroll
+    for (int n1 = 0; n1 < A; ++n1) t[n2][n1] = v[(B * n1 + A * n2) % (A * B)];
+    dft_small<A, INV>(t[n2]);
+  }
+#pragma unroll
+  for (int k1 = 0; k1 < A; ++k1) {
+    C u[B];
+#pragma unroll
+    for (int n2 = 0; n2 < B; ++n2) u[n2] = t[n2][k1];
+    dft_small<B, INV>(u);
+#pragma unroll
+    for (int k2 = 0; k2 < B; ++k2) v[(EA * k1 + EB * k2) % (A * B)] = u[k2];
+  }
+}
 template <int RAD, bool INV, typename C> __device__ __forceinline__ void dft(C *v) {
   if constexpr (RAD == 2) dft2<INV>(v);
   else if constexpr (RAD == 3) dft3<INV>(v);
   else if constexpr (RAD == 4) dft4<INV>(v);
   else if constexpr (RAD == 5) dft5<INV>(v);
   else if constexpr (RAD == 8) dft8<INV>(v);
+  else if constexpr (RAD == 12) dft_pf<3, 4, 4, 9, INV>(v);  // 4 = 1 mod 3, 9 = 1 mod 4
   else if constexpr (RAD == 16) dft16<INV>(v);
+  else if constexpr (RAD == 20) dft_pf<4, 5, 5, 16, INV>(v);  // 5 = 1 mod 4, 16 = 1 mod 5
 }
 
 // ------------------------------------ FMA form of a twiddled radix-2^L DFT

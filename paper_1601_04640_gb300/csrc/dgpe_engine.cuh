@@ -247,10 +247,14 @@ template <typename R> struct EngineT : Engine {
   bool p1_pipe = false;
   int p1_grid[2] = {0, 0};  // real, complex CN coefficients
   size_t p1_smem[2] = {0, 0};
-  // ... and the pipelined density / R2C pass (k_p4_pipe)
-  bool p4_pipe = false;
-  int p4_grid = 0;
-  size_t p4_smem = 0;
+  // FP32 bulk: the warp-per-tile x-row passes (dgpe_rows*.cu); persistent
+  // grids by forward source and backward mode (ROWS_STEP: imaginary time
+  // first, real time last), constant CN forms along x, tensor map of psi
+  bool rows_fwd = false, rows_back = false;
+  int rows_fgrid[3] = {0, 0, 0}, rows_bgrid[ROWS_MODES + 1] = {0};
+  CnConst<float> row_kr{};
+  CnConst<float2> row_kc{}, row_ka{};
+  CUtensorMap tm_psi{};
   // ... and the TMA-tiled strided transforms (k_fft_tma): tensor maps of the
   // half spectrum for lines along y and along z
   bool tma_fft = false;
@@ -631,6 +635,12 @@ template <typename R> struct EngineT : Engine {
         if (dl >= 64) dl = 0;
       }
       cn_dlim[a] = dl;
+      if (a == 0 && sizeof(R) == 4) {
+        const int cl = rows_chunk(n);
+        row_kr = cn_const<float>(zd(tau[0], 0.0), cl, n / cl);
+        row_kc = cn_const<float2>(zd(0.0, tau[0]), cl, n / cl);
+        row_ka = cn_const<float2>(zd(0.0, -tau[0]), cl, n / cl);
+      }
       cn_kr[a] = cn_const<float>(zd(tau[a], 0.0), C, n / C);
       cn_kc[a] = cn_const<float2>(zd(0.0, tau[a]), C, n / C);
       cn_ka[a] = cn_const<float2>(zd(0.0, -tau[a]), C, n / C);
@@ -735,26 +745,6 @@ template <typename R> struct EngineT : Engine {
           });
           if (r) return r;
         }
-        p4_pipe = !rpsi && !(p.flags & DGPE_FLAG_P1_ONESHOT);
-        if (p4_pipe) {
-          p4_smem = sizeof(Cx) * (2 * (size_t)2 * x_LP * nx + (size_t)x_LP * x_pitchz);
-          r = with_pow2_len(nx, [&](auto Nc) -> int {
-            constexpr int N = decltype(Nc)::value;
-            if constexpr (N == 0 || CL != 16) {
-              p4_pipe = false;
-              return DGPE_OK;
-            } else {
-              int q;
-              if ((q = smem_attr(k_p4_pipe<EX, N>, p4_smem))) return q;
-              int occ = 0;
-              DGPE_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_p4_pipe<EX, N>, x_T, p4_smem));
-              if (occ < 1) p4_pipe = false;
-              p4_grid = std::max(1, std::min(x_grid, nsm * occ));
-              return DGPE_OK;
-            }
-          });
-          if (r) return r;
-        }
       }
       return DGPE_OK;
     });
@@ -795,9 +785,37 @@ template <typename R> struct EngineT : Engine {
       });
       if (rc) return rc;
     }
+    if ((rc = setup_rows())) return rc;
     return setup_tma();
   }
 
+  // The state (nx reals or complex per row) as rows of 16 elements, boxes of
+  // 64 of them (a warp's tile), swizzled so that a lane's 16-byte pieces lie
+  // on the banks its neighbours' do not (dgpe_rows_back.cuh).
+  bool row_map(CUtensorMap *tm, void *buf) {
+    TensorMapEncodeTiledFn enc = tensor_map_encoder();
+    if (!enc) return false;
+    const cuuint64_t dims[2] = {16, (cuuint64_t)(nsites / 16)}, strides[1] = {rpsi ? 64u : 128u};
+    const cuuint32_t box[2] = {16, 64}, es[2] = {1, 1};
+    return enc(tm, rpsi ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, buf, dims, strides, box, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, rpsi ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  }
+  int setup_rows() {
+    if constexpr (sizeof(R) == 4) {
+      if (p.flags & DGPE_FLAG_P1_ONESHOT) return DGPE_OK;
+      if (has_dip) {
+        for (int k = 0; k < 3; ++k) DGPE_CK(rows_fwd_grid(nx, nrows, k, nsm, &rows_fgrid[k]));
+        rows_fwd = true;
+      }
+      if (!row_map(&tm_psi, psi)) return DGPE_OK;
+      for (int m : {ROWS_STEP, ROWS_PHI, ROWS_REAL}) DGPE_CK(rows_back_grid_real(nx, nrows, m, nsm, &rows_bgrid[m]));
+      for (int m : {ROWS_CN, ROWS_EXP}) DGPE_CK(rows_back_grid_cplx(nx, nrows, m, nsm, &rows_bgrid[m]));
+      DGPE_CK(rows_back_grid_cplx(nx, nrows, ROWS_STEP, nsm, &rows_bgrid[ROWS_MODES]));
+      rows_back = true;
+    }
+    return DGPE_OK;
+  }
   // Persistent grids of the register-resident line passes for the current mode.
   void setup_lines() {
     if constexpr (sizeof(R) == 4) {
@@ -1011,6 +1029,60 @@ template <typename R> struct EngineT : Engine {
     }
     return DGPE_OK;
   }
+  // FP32: the x-row passes; false where another kernel has to run (the
+  // one-shot flag, slowly decaying coefficients, a caller's buffer that the
+  // bulk copies cannot start at).
+  static bool aligned16(const void *ptr) { return ((uintptr_t)ptr & 15) == 0; }
+  RowArgs rargs() const {
+    RowArgs A{};
+    if constexpr (sizeof(R) == 4) {
+      A.psi = psi; A.spec = spec; A.phi_out = phi_tmp; A.prm = prm; A.step = dstep;
+      A.tw = tw[0]; A.vx = vt[0]; A.vy = vt[1]; A.vz = vt[2];
+      A.n = nx; A.ny = ny; A.nrows = nrows; A.has_dip = has_dip ? 1 : 0; A.dtf = 1.0;
+    }
+    return A;
+  }
+  bool launch_rows_fwd(cudaStream_t s, const Cx *src, const R *dens_in, cudaError_t &e) {
+    if constexpr (sizeof(R) == 4) {
+      if (!rows_fwd || (src && !aligned16(src)) || (dens_in && !aligned16(dens_in))) return false;
+      RowArgs A = rargs();
+      if (src) A.psi = const_cast<Cx *>(src);
+      A.dens_in = dens_in;
+      A.src = dens_in ? 1 : (rpsi && !src) ? 2 : 0;
+      e = rows_fwd_launch(A, rows_fgrid[A.src], s);
+      return true;
+    }
+    return false;
+  }
+  bool launch_rows_back(int mode, cudaStream_t s, Cx *buf, R *phi_out, double dtf, cudaError_t &e) {
+    if constexpr (sizeof(R) == 4) {
+      if (!rows_back) return false;
+      static const int modes[4] = {ROWS_STEP, ROWS_PHI, ROWS_CN, ROWS_EXP};
+      RowArgs A = rargs();
+      A.mode = (mode == 0 && rpsi) ? (int)ROWS_REAL : modes[mode];
+      A.dtf = dtf;
+      if (phi_out) A.phi_out = phi_out;
+      if (A.mode == ROWS_PHI) {
+        e = rows_back_launch(A, tm_psi, row_kr, rows_bgrid[ROWS_PHI], s);
+        return true;
+      }
+      if (imag) {
+        if (mode != 0 || row_kr.dl == 0) return false;
+        e = rows_back_launch(A, tm_psi, row_kr, rows_bgrid[A.mode], s);
+        return true;
+      }
+      const CnConst<float2> &K = mode == 2 ? row_ka : row_kc;
+      if (K.dl == 0 && mode != 3) return false;
+      CUtensorMap tm = tm_psi;
+      if (buf && buf != psi) {
+        if (!aligned16(buf) || !row_map(&tm, buf)) return false;
+        A.psi = buf;
+      }
+      e = rows_back_launch(A, tm, K, rows_bgrid[A.mode == ROWS_STEP ? (int)ROWS_MODES : A.mode], s);
+      return true;
+    }
+    return false;
+  }
   int launch_cn(int axis, bool final_pass, cudaStream_t s, Cx *buf = nullptr, bool adjoint = false) {
     if (cn_serial) return launch_lines(axis, final_pass, s, buf, adjoint);
     if constexpr (sizeof(R) == 4) return launch_cols(axis, final_pass, s, buf, adjoint);
@@ -1052,6 +1124,12 @@ template <typename R> struct EngineT : Engine {
   }
   // density (of `src`, or the real field `dens_in`) -> half spectrum along x
   int launch_forward_spectrum(cudaStream_t s, const Cx *src = nullptr, const R *dens_in = nullptr) {
+    cudaError_t e = cudaSuccess;
+    if (launch_rows_fwd(s, src, dens_in, e)) {
+      launched(1);
+      DGPE_CK(e);
+      return DGPE_OK;
+    }
     XArgs<R> A = xargs();
     if (src) A.psi = const_cast<Cx *>(src);
     if (dens_in) A.dens_in = dens_in;
@@ -1062,15 +1140,7 @@ template <typename R> struct EngineT : Engine {
       constexpr bool FM1 = P2 && sizeof(R) == 8;  // the C2R pass: FP64 only
       if (dens_in) k_dens_r2c_x<R, EX, 1, P2, FM><<<x_grid, x_T, x4_smem, s>>>(A);
       else if (rpsi && !src) k_dens_r2c_x<R, EX, 2, P2, FM><<<x_grid, x_T, x4_smem, s>>>(A);
-      else if (p4_pipe) {
-        if constexpr (sizeof(R) == 4 && P2 && decltype(CLc)::value == 16) {
-          with_pow2_len(nx, [&](auto Nc) -> int {
-            constexpr int N = decltype(Nc)::value;
-            if constexpr (N != 0) k_p4_pipe<EX, N><<<p4_grid, x_T, p4_smem, s>>>(A, x_grid, prm + PRM_TIMEOUT);
-            return 0;
-          });
-        }
-      } else k_dens_r2c_x<R, EX, 0, P2, FM><<<x_grid, x_T, x4_smem, s>>>(A);
+      else k_dens_r2c_x<R, EX, 0, P2, FM><<<x_grid, x_T, x4_smem, s>>>(A);
       return DGPE_OK;
     });
     launched(1);
@@ -1082,6 +1152,12 @@ template <typename R> struct EngineT : Engine {
   // exponential over the fraction dtf of dt
   int launch_p1(int mode, cudaStream_t s, Cx *buf = nullptr, R *phi_out = nullptr, double dtf = 1.0) {
     if (mode == 2 && cn_serial) return launch_lines(0, false, s, buf, true);
+    cudaError_t e = cudaSuccess;
+    if (launch_rows_back(mode, s, buf, phi_out, dtf, e)) {
+      launched(1);
+      DGPE_CK(e);
+      return DGPE_OK;
+    }
     XArgs<R> A = xargs();
     A.dtf = dtf;
     if (buf) A.psi = buf;

@@ -547,94 +547,6 @@ __global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB_P1(R)) k_c2r_x_exp_cnx_ba
 #define DGPE_WAIT_LIMIT (1 << 22)  // polls of a bounded mbarrier wait
 #endif
 
-// ----------------------------------------------- P4, FP32 pipelined form
-// The density + R2C pass of the FP32 bulk (complex state, power-of-two nx) as
-// a persistent pipeline: a tile's 2 LP rows of psi are one contiguous block,
-// brought into one of two staging buffers by a bulk copy on that buffer's
-// mbarrier, two tiles ahead of the transform.  The density is formed as the
-// first Stockham stage reads the staged rows; the separated half spectra are
-// stored from the Z tile.  Shared memory (dynamic): 2 psi stages [2 LP][nx],
-// Z tile [LP][pitchz].
-template <int EPT, int N>
-__global__ void __launch_bounds__(DGPE_MAXT, 2) k_p4_pipe(const __grid_constant__ XArgs<float> A, int ntiles,
-                                                         double *timeout_flag) {
-  typedef float R;
-  typedef float2 Cx;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int PW = Pad<R>::W;
-  constexpr int T = DGPE_MAXT, TPL = N / 16, LP = (DGPE_MAXT / 2) / TPL, ROWS = 2 * LP;
-  constexpr int SL = N + N / PW + 1, PX = N / 2 + 2, LN = ct_log2(N), NH = N / 2 + 1;
-  const int nrows = A.nrows;
-  const int t = threadIdx.x;
-  Cx *const stg0 = reinterpret_cast<Cx *>(smraw);  // stage k at stg0 + k ROWS N
-  Cx *const zt = reinterpret_cast<Cx *>(smraw) + 2 * ROWS * N;
-  __shared__ unsigned long long bar[2];
-  __shared__ R s_sc2;
-  __shared__ __align__(16) Cx s_tw[N];
-  auto issue = [&](int tile, int k) {  // thread 0
-    const int r0 = tile * ROWS;
-    const int nr = (nrows - r0 < ROWS) ? nrows - r0 : ROWS;
-    const unsigned bp = (unsigned)(sizeof(Cx) * (size_t)nr * N);
-    fence_proxy_async_smem();
-    mbar_expect_tx(&bar[k], bp);
-    bulk_g2s(stg0 + k * ROWS * N, A.psi + (size_t)r0 * N, bp, &bar[k]);
-  };
-  if (t == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
-    const R sc = (R)A.prm[PRM_SC];
-    s_sc2 = sc * sc;
-  }
-  __syncthreads();
-  if (t == 0) {
-    if ((int)blockIdx.x < ntiles) issue(blockIdx.x, 0);
-    if ((int)(blockIdx.x + gridDim.x) < ntiles) issue(blockIdx.x + gridDim.x, 1);
-  }
-  for (int i = t; i < N; i += T) s_tw[i] = A.tw[i];
-  __syncthreads();
-  const R sc2 = s_sc2;
-  unsigned ph = 0u;  // bit k: the phase parity stage k waits for next
-  int k = 0;
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, k ^= 1) {
-    const int r0 = tile * ROWS;
-    const bool ok = mbar_wait_bounded(&bar[k], (ph >> k) & 1u, DGPE_WAIT_LIMIT);
-    ph ^= 1u << k;
-    if (__syncthreads_or(!ok)) {
-      if (t == 0) {
-        // the copy into the other stage, if one was issued, lands (bounded wait) before the block exits
-        if (tile + (int)gridDim.x < ntiles) mbar_wait_bounded(&bar[k ^ 1], (ph >> (k ^ 1)) & 1u, DGPE_WAIT_LIMIT);
-        *timeout_flag = 1.0;
-      }
-      return;
-    }
-    const Cx *__restrict__ sp = stg0 + k * ROWS * N;
-    const bool full = (r0 + ROWS <= nrows);
-    auto load = [&](int l, int a) -> cx<R> {
-      R d0 = 0, d1 = 0;
-      if (full || r0 + 2 * l < nrows) { const Cx v = sp[((2 * l) << LN) + a]; d0 = sc2 * (v.x * v.x + v.y * v.y); }
-      if (full || r0 + 2 * l + 1 < nrows) { const Cx v = sp[((2 * l + 1) << LN) + a]; d1 = sc2 * (v.x * v.x + v.y * v.y); }
-      return mk<R>(d0, d1);
-    };
-    auto store = [&](int l, int a, cx<R> v) { zt[l * SL + a + a / PW] = v; };
-    tile_fft_ct<R, N, EPT, false, PW, SL, LP, T>(zt, s_tw, load, store);
-    // this stage is consumed: refill it two tiles ahead
-    const int next2 = tile + 2 * gridDim.x;
-    if (t == 0 && next2 < ntiles) issue(next2, k);
-    // two real lines were packed as Z = n0 + i n1
-    for (int idx = t; idx < LP * NH; idx += T) {
-      const int l = idx / NH, kk = idx - l * NH;
-      const int ra = r0 + 2 * l, rb = ra + 1;
-      if (ra >= nrows) continue;
-      const int km = (kk == 0 ? 0 : N - kk);
-      const cx<R> Zk = zt[l * SL + kk + kk / PW], Zm = zt[l * SL + km + km / PW];
-      A.spec[(size_t)ra * PX + kk] = mk<R>((R)0.5 * (Zk.x + Zm.x), (R)0.5 * (Zk.y - Zm.y));
-      if (rb < nrows) A.spec[(size_t)rb * PX + kk] = mk<R>((R)0.5 * (Zk.y + Zm.y), (R)0.5 * (Zm.x - Zk.x));
-    }
-  }
-  __syncthreads();
-  if (t == 0) { mbar_inval(&bar[0]); mbar_inval(&bar[1]); }
-}
-
 // ----------------------------------------------- P1, FP32 pipelined form
 // The x-line pass of the FP32 bulk (complex state, power-of-two nx) as a
 // persistent pipeline.  A tile is the 2 LP consecutive rows of psi and of the

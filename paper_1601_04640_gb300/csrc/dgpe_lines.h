@@ -1,9 +1,10 @@
 // dgpe_lines.h -- arguments and launchers of the register-resident line
-// passes of the FP32 bulk (dgpe_rows.cu: x-rows; dgpe_cols.cu: the strided
+// passes of the FP32 bulk (dgpe_rows*.cu: x-rows; dgpe_cols.cu: the strided
 // Crank-Nicolson solves along y and z).  Each kernel is compiled once, in
 // those units; the solver and the batched form call the launchers.
 #pragma once
 
+#include <cuda.h>  // CUtensorMap
 #include <cuda_runtime.h>
 
 namespace dgpe {
@@ -13,7 +14,7 @@ namespace dgpe {
 // reach dl of the chunk inflow (1..4 chunks; 0: the coefficients decay too
 // slowly for this form) and the number J <= CL of sites of a chunk that an
 // inflow still changes.
-enum { CN_PW = 16, CN_DL = 4 };
+enum { CN_PW = 20, CN_DL = 4 };
 template <typename Coef> struct CnConst {
   Coef al, m2, pc, pw[CN_PW];
   int dl, J;
@@ -41,8 +42,8 @@ int cols_grid(int n, int cl, unsigned tot, int nsm, bool real_coef, bool tab);
 cudaError_t cols_launch(const ColArgs &A, const CnConst<float> &K, int grid, cudaStream_t s);
 cudaError_t cols_launch(const ColArgs &A, const CnConst<float2> &K, int grid, cudaStream_t s);
 
-// x-row passes.  psi: [nrows][n] complex (src 2 / mode 4: real); spec: the half
-// spectrum, rows of px elements.
+// x-row passes (dgpe_rows*.cu).  psi: [nrows][n] complex (src 2 / ROWS_REAL:
+// real), 16-byte aligned; spec: the half spectrum, rows of n / 2 + 2 elements.
 struct RowArgs {
   float2 *psi;
   float2 *spec;
@@ -52,20 +53,24 @@ struct RowArgs {
   const long long *step;
   const float2 *tw;  // exp(-2 pi i t / n)
   const float *vx, *vy, *vz;
-  int n, ny, nrows, px;
-  int has_dip, imag;
-  int src;   // forward: 0 sc^2 |psi|^2, 1 the real field dens_in, 2 sc^2 psi^2 of a real state
-  int mode;  // backward: ROWS_*
+  int n, ny, nrows;
+  int has_dip;
+  int src;     // forward: 0 sc^2 |psi|^2, 1 the real field dens_in, 2 sc^2 psi^2 of a real state
+  int mode;    // backward: ROWS_*
   double dtf;  // fraction of dt of the exponential substep
 };
-enum { ROWS_STEP = 0, ROWS_PHI = 1, ROWS_CN = 2, ROWS_EXP = 3, ROWS_REAL = 4 };
-// density + R2C along x
-int rows_fwd_grid(int n, int nrows, int nsm);
+// C2R along x, exponential, Crank-Nicolson along x (STEP; REAL: of a real
+// state), or one of them alone (PHI: Phi_d into phi_out; CN; EXP)
+enum { ROWS_STEP = 0, ROWS_PHI = 1, ROWS_CN = 2, ROWS_EXP = 3, ROWS_REAL = 4, ROWS_MODES = 5 };
+// points of a row that one lane solves: the chunk length of the constant form
+int rows_chunk(int n);
+// The grids raise the kernels' shared-memory limits: once before a launch.
+cudaError_t rows_fwd_grid(int n, int nrows, int src, int nsm, int *grid);
 cudaError_t rows_fwd_launch(const RowArgs &A, int grid, cudaStream_t s);
-// C2R along x, exponential, Crank-Nicolson along x (modes STEP, REAL), or one
-// of them alone (PHI: Phi_d into phi_out; CN; EXP)
-int rows_back_grid(int n, int nrows, int nsm, bool real_coef, bool real_state);
-cudaError_t rows_back_launch(const RowArgs &A, const CnConst<float> &K, int grid, cudaStream_t s);
-cudaError_t rows_back_launch(const RowArgs &A, const CnConst<float2> &K, int grid, cudaStream_t s);
+// tm: the state as rows of 16 elements (2^k lengths; see rows_back.cuh)
+cudaError_t rows_back_grid_real(int n, int nrows, int mode, int nsm, int *grid);
+cudaError_t rows_back_grid_cplx(int n, int nrows, int mode, int nsm, int *grid);
+cudaError_t rows_back_launch(const RowArgs &A, const CUtensorMap &tm, const CnConst<float> &K, int grid, cudaStream_t s);
+cudaError_t rows_back_launch(const RowArgs &A, const CUtensorMap &tm, const CnConst<float2> &K, int grid, cudaStream_t s);
 
 }  // namespace dgpe
