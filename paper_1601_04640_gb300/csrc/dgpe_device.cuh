@@ -453,6 +453,16 @@ constexpr int ct_nstages(int n, int ept) {
   while (m > 1) { m /= ct_radix(n, ept, s); ++s; }
   return s;
 }
+// The solver's column tiles take a first stage of 12 (3 2^k) or 20 (5 2^k)
+// points when a thread holds as many: one stage fewer.
+constexpr bool ct_first_pf(int n, int ept) { return (ept == 12 || ept == 20) && n % ept == 0; }
+constexpr int ct_radix_cols(int n, int ept, int s) {
+  if (!ct_first_pf(n, ept)) return ct_radix(n, ept, s);
+  return s == 0 ? ept : ct_radix(n / ept, ept, s - 1);
+}
+constexpr int ct_nstages_cols(int n, int ept) {
+  return ct_first_pf(n, ept) ? 1 + ct_nstages(n / ept, ept) : ct_nstages(n, ept);
+}
 constexpr int ct_log2(int v) { return v <= 1 ? 0 : 1 + ct_log2(v / 2); }
 
 // LINE_FAST: consecutive threads take consecutive lines (column tiles, element
@@ -521,25 +531,26 @@ __device__ __forceinline__ void fft_stage_ct(cx<R> *sm, const cx<R> *__restrict_
   __syncthreads();
 }
 template <typename R, int N, int EPT, bool INV, int PADW, int SL, int NL, int T, bool LINE_FAST, int SA, int S,
-          int NSACC, class Load, class Store>
+          int NSACC, bool PF, class Load, class Store>
 __device__ __forceinline__ void tile_fft_ct_from(cx<R> *sm, const cx<R> *__restrict__ tw, Load &load, Store &store) {
-  constexpr int NST = ct_nstages(N, EPT);
+  constexpr int NST = PF ? ct_nstages_cols(N, EPT) : ct_nstages(N, EPT);
   if constexpr (S < NST) {
-    constexpr int RAD = INV ? ct_radix(N, EPT, NST - 1 - S) : ct_radix(N, EPT, S);
+    constexpr int K = INV ? NST - 1 - S : S, RAD = PF ? ct_radix_cols(N, EPT, K) : ct_radix(N, EPT, K);
     fft_stage_ct<R, N, EPT, RAD, NSACC, INV, PADW, SL, NL, T, S == 0, S == NST - 1, LINE_FAST, SA>(sm, tw, load,
                                                                                                   store);
-    tile_fft_ct_from<R, N, EPT, INV, PADW, SL, NL, T, LINE_FAST, SA, S + 1, NSACC * RAD>(sm, tw, load, store);
+    tile_fft_ct_from<R, N, EPT, INV, PADW, SL, NL, T, LINE_FAST, SA, S + 1, NSACC * RAD, PF>(sm, tw, load, store);
   }
 }
 // Full transform of the NL lines of a line-major tile; tw[t] = exp(-2 pi i t / N).
 template <typename R, int N, int EPT, bool INV, int PADW, int SL, int NL, int T, class Load, class Store>
 __device__ __forceinline__ void tile_fft_ct(cx<R> *sm, const cx<R> *__restrict__ tw, Load load, Store store) {
-  tile_fft_ct_from<R, N, EPT, INV, PADW, SL, NL, T, false, 1, 0, 1>(sm, tw, load, store);
+  tile_fft_ct_from<R, N, EPT, INV, PADW, SL, NL, T, false, 1, 0, 1, false>(sm, tw, load, store);
 }
 // ... of a column tile of NL lines (element a of line l at a NL + l).
-template <typename R, int N, int EPT, bool INV, int NL, int T, class Load, class Store>
+// PF: with a 12- or 20-point first stage (ct_radix_cols).
+template <typename R, int N, int EPT, bool INV, int NL, int T, bool PF = false, class Load, class Store>
 __device__ __forceinline__ void tile_fft_ct_cols(cx<R> *sm, const cx<R> *__restrict__ tw, Load load, Store store) {
-  tile_fft_ct_from<R, N, EPT, INV, 0, 1, NL, T, true, NL, 0, 1>(sm, tw, load, store);
+  tile_fft_ct_from<R, N, EPT, INV, 0, 1, NL, T, true, NL, 0, 1, PF>(sm, tw, load, store);
 }
 
 // ------------------------------------------- Crank-Nicolson (Thomas) solve

@@ -197,6 +197,20 @@ template <class F> int with_pow2_len(int n, F &&f) {
   }
 }
 
+// Call f(N, EPT) for any line length of the FP32 strided transforms (EPT
+// elements per thread: 16, 12 or 20 for 2^k, 3 2^k, 5 2^k).
+template <class F> int with_col_len(int n, F &&f) {
+  switch (n) {
+#define DGPE_COL(N) \
+  case N: return f(std::integral_constant<int, N>{}, std::integral_constant<int, N % 3 == 0 ? 12 : N % 5 == 0 ? 20 : 16>{});
+    DGPE_COL(32) DGPE_COL(64) DGPE_COL(128) DGPE_COL(256) DGPE_COL(512)
+    DGPE_COL(48) DGPE_COL(96) DGPE_COL(192) DGPE_COL(384)
+    DGPE_COL(40) DGPE_COL(80) DGPE_COL(160) DGPE_COL(320)
+#undef DGPE_COL
+    default: return DGPE_EUNSUPPORTED;
+  }
+}
+
 template <typename R> struct EngineT : Engine {
   typedef cx<R> Cx;
   static constexpr int EPT_S = sizeof(R) == 8 ? DGPE_EPT_S_F64 : 16;  // strided FFTs, power-of-two lengths
@@ -850,65 +864,53 @@ template <typename R> struct EngineT : Engine {
     A.uny = ny;
     return A;
   }
-  // FP32, power-of-two length, modes 0-2: the length-specialised transform
+  // FP32, modes 0-2: the length-specialised transform fed by registers
   bool launch_fft_ct(const FtCfg &f, int mode, const SArgs<R> &A, cudaStream_t s) {
     if constexpr (sizeof(R) != 4) {
       return false;
     } else {
-      if (mode > 2 || var[f.axis] != VAR_P2 || !(f.W == 16 || f.W == 8 || f.W == 4)) return false;
-      return with_pow2_len(f.n, [&](auto Nc) -> int {
-        constexpr int N = decltype(Nc)::value;
-        if constexpr (N == 0) {
-          return 0;
-        } else {
-          auto go = [&](auto Wc) {
-            constexpr int WW = decltype(Wc)::value;
-            if constexpr (WW * N / EPT_S <= DGPE_MAXT_FFT) {
-              if (mode == 0) k_fft_strided_ct<EPT_S, 0, N, WW><<<f.grid, f.T, f.smem, s>>>(A);
-              else if (mode == 1) k_fft_strided_ct<EPT_S, 1, N, WW><<<f.grid, f.T, f.smem, s>>>(A);
-              else k_fft_strided_ct<EPT_S, 2, N, WW><<<f.grid, f.T, f.smem, s>>>(A);
-              return 1;
-            } else {
-              return 0;
-            }
-          };
-          if (f.W == 16) return go(std::integral_constant<int, 16>{});
-          if (f.W == 8) return go(std::integral_constant<int, 8>{});
-          return go(std::integral_constant<int, 4>{});
-        }
-      }) != 0;
+      if (mode > 2) return false;
+      bool done = false;
+      with_col_len(f.n, [&](auto Nc, auto Ec) -> int {
+        constexpr int N = decltype(Nc)::value, E = decltype(Ec)::value, WW = col_width(N, E);
+        if (f.W != WW) return 0;
+        if (mode == 0) k_fft_strided_ct<E, 0, N, WW><<<f.grid, f.T, f.smem, s>>>(A);
+        else if (mode == 1) k_fft_strided_ct<E, 1, N, WW><<<f.grid, f.T, f.smem, s>>>(A);
+        else k_fft_strided_ct<E, 2, N, WW><<<f.grid, f.T, f.smem, s>>>(A);
+        done = true;
+        return 0;
+      });
+      return done;
     }
   }
-  // FP32, power-of-two lengths: tensor maps of the half spectrum (kx, y, z;
-  // kx valid columns, rows of px elements) for the TMA-tiled transforms.
-  // Not fatal when unavailable: the length-specialised kernels run instead.
+  // Tile width of a strided FP32 transform: DGPE_W_FFT_F32 columns, halved
+  // until a block has at most DGPE_MAXT_FFT threads.
+  static constexpr int col_width(int n, int ept) {
+    int w = DGPE_W_FFT_F32;
+    while (w > 1 && w * n / ept > DGPE_MAXT_FFT) w >>= 1;
+    return w;
+  }
+  // FP32: tensor maps of the half spectrum (kx, y, z; kx valid columns, rows
+  // of px elements) for the TMA-tiled transforms.  Not fatal when
+  // unavailable: the length-specialised kernels run instead.
   int tma_grid[2] = {0, 0};
-  template <int AX, int N, int WW> int tma_attrs(int &grid) {
+  template <int AX, int N, int E> int tma_attrs(int &grid) {
+    constexpr int WW = col_width(N, E);
     const size_t sm = 2 * sizeof(Cx) * (size_t)WW * N + 128;
     int r;
     if constexpr (AX == 1) {  // lines along y: FFT_y, IFFT_y (3D) and FFT_y.U.IFFT_y (2D)
-      if ((r = smem_attr(k_fft_tma<EPT_S, 0, N, WW, AX>, sm))) return r;
-      if ((r = smem_attr(k_fft_tma<EPT_S, 1, N, WW, AX>, sm))) return r;
+      if ((r = smem_attr(k_fft_tma<E, 0, N, WW, AX>, sm))) return r;
+      if ((r = smem_attr(k_fft_tma<E, 1, N, WW, AX>, sm))) return r;
     }
-    if ((r = smem_attr(k_fft_tma<EPT_S, 2, N, WW, AX>, sm))) return r;
+    if ((r = smem_attr(k_fft_tma<E, 2, N, WW, AX>, sm))) return r;
     int occ = 0;
-    DGPE_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_fft_tma<EPT_S, 2, N, WW, AX>, WW * N / EPT_S, sm));
+    DGPE_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_fft_tma<E, 2, N, WW, AX>, WW * N / E, sm));
     grid = nsm * occ;
     return DGPE_OK;
   }
   template <int AX> int tma_axis(const FtCfg &f, int &grid) {
-    return with_pow2_len(f.n, [&](auto Nc) -> int {
-      constexpr int N = decltype(Nc)::value;
-      if constexpr (N == 0) {
-        return DGPE_EUNSUPPORTED;
-      } else {
-        if (f.W == 16) {
-          if constexpr (16 * N / EPT_S <= DGPE_MAXT_FFT) return this->template tma_attrs<AX, N, 16>(grid);
-        } else if (f.W == 8) {
-          if constexpr (8 * N / EPT_S <= DGPE_MAXT_FFT) return this->template tma_attrs<AX, N, 8>(grid);
-        }
-        return DGPE_EUNSUPPORTED;
-      }
+    return with_col_len(f.n, [&](auto Nc, auto Ec) -> int {
+      return this->template tma_attrs<AX, decltype(Nc)::value, decltype(Ec)::value>(grid);
     });
   }
   int setup_tma() {
@@ -917,7 +919,6 @@ template <typename R> struct EngineT : Engine {
     } else {
       tma_fft = false;
       if (!has_dip || (p.flags & DGPE_FLAG_P1_ONESHOT)) return DGPE_OK;
-      if (var[1] != VAR_P2 || (dim == 3 && var[2] != VAR_P2)) return DGPE_OK;
       TensorMapEncodeTiledFn enc = tensor_map_encoder();
       if (!enc) return DGPE_OK;
       const cuuint64_t dims[3] = {(cuuint64_t)ncol_spec, (cuuint64_t)ny, (cuuint64_t)nz};
@@ -937,12 +938,10 @@ template <typename R> struct EngineT : Engine {
           return DGPE_OK;
       }
       int r = this->template tma_axis<1>(fy, tma_grid[0]);
-      if (r == DGPE_EUNSUPPORTED) return DGPE_OK;
       if (r) return r;
       if (dim == 3) {
         r = this->template tma_axis<2>(fz, tma_grid[1]);
-        if (r == DGPE_EUNSUPPORTED) return DGPE_OK;
-        if (r) return r;
+          if (r) return r;
       }
       tma_fft = tma_grid[0] > 0 && (dim == 2 || tma_grid[1] > 0);
       return DGPE_OK;
@@ -952,39 +951,20 @@ template <typename R> struct EngineT : Engine {
     if constexpr (sizeof(R) != 4) {
       return false;
     } else {
-      if (!tma_fft || mode > 2) return false;
+      if (!tma_fft || mode > 2 || (f.axis == 2 && mode != 2)) return false;
       const int ncb = (int)f.grid.x, ntiles = (int)(f.grid.x * f.grid.y);
-      return with_pow2_len(f.n, [&](auto Nc) -> int {
-        constexpr int N = decltype(Nc)::value;
-        if constexpr (N == 0) {
-          return 0;
-        } else {
-          auto go = [&](auto Wc) -> int {
-            constexpr int WW = decltype(Wc)::value;
-            if constexpr (WW * N / EPT_S <= DGPE_MAXT_FFT) {
-              const size_t sm = 2 * sizeof(Cx) * (size_t)WW * N + 128;
-              const int T = WW * N / EPT_S;
-              double *tf = prm + PRM_TIMEOUT;
-              if (f.axis == 1) {
-                const int g = std::max(1, std::min(ntiles, tma_grid[0]));
-                if (mode == 0) k_fft_tma<EPT_S, 0, N, WW, 1><<<g, T, sm, s>>>(tm_y, A, ncb, ntiles, tf);
-                else if (mode == 1) k_fft_tma<EPT_S, 1, N, WW, 1><<<g, T, sm, s>>>(tm_y, A, ncb, ntiles, tf);
-                else k_fft_tma<EPT_S, 2, N, WW, 1><<<g, T, sm, s>>>(tm_y, A, ncb, ntiles, tf);
-              } else {
-                const int g = std::max(1, std::min(ntiles, tma_grid[1]));
-                if (mode != 2) return 0;
-                k_fft_tma<EPT_S, 2, N, WW, 2><<<g, T, sm, s>>>(tm_z, A, ncb, ntiles, tf);
-              }
-              return 1;
-            } else {
-              return 0;
-            }
-          };
-          if (f.W == 16) return go(std::integral_constant<int, 16>{});
-          if (f.W == 8) return go(std::integral_constant<int, 8>{});
-          return 0;
-        }
-      }) != 0;
+      const int g = std::max(1, std::min(ntiles, tma_grid[f.axis - 1]));
+      double *tf = prm + PRM_TIMEOUT;
+      with_col_len(f.n, [&](auto Nc, auto Ec) -> int {
+        constexpr int N = decltype(Nc)::value, E = decltype(Ec)::value, WW = col_width(N, E), T = WW * N / E;
+        const size_t sm = 2 * sizeof(Cx) * (size_t)WW * N + 128;
+        if (f.axis == 2) k_fft_tma<E, 2, N, WW, 2><<<g, T, sm, s>>>(tm_z, A, ncb, ntiles, tf);
+        else if (mode == 0) k_fft_tma<E, 0, N, WW, 1><<<g, T, sm, s>>>(tm_y, A, ncb, ntiles, tf);
+        else if (mode == 1) k_fft_tma<E, 1, N, WW, 1><<<g, T, sm, s>>>(tm_y, A, ncb, ntiles, tf);
+        else k_fft_tma<E, 2, N, WW, 1><<<g, T, sm, s>>>(tm_y, A, ncb, ntiles, tf);
+        return 0;
+      });
+      return true;
     }
   }
   int launch_fft(const FtCfg &f, int mode, cudaStream_t s) {

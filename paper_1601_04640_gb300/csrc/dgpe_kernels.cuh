@@ -806,17 +806,17 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, DGPE_MINB_FFT_F32) k_fft_stride
     if (fullw || c0 + l < A.ncols) spec[base + a * es + l] = v;
   };
   if constexpr (MODE == 0) {
-    tile_fft_ct_cols<R, N, EPT, false, W, T>(sm, s_tw, gload, gstore);
+    tile_fft_ct_cols<R, N, EPT, false, W, T, true>(sm, s_tw, gload, gstore);
   } else if constexpr (MODE == 1) {
-    tile_fft_ct_cols<R, N, EPT, true, W, T>(sm, s_tw, gload, gstore);
+    tile_fft_ct_cols<R, N, EPT, true, W, T, true>(sm, s_tw, gload, gstore);
   } else {
     auto mstore = [&](int l, int a, Cx v) {
       const R u = (fullw || c0 + l < A.ncols) ? A.U[base + a * es + l] : (R)0;
       sm[a * W + l] = cscale(v, u);
     };
-    tile_fft_ct_cols<R, N, EPT, false, W, T>(sm, s_tw, gload, mstore);
+    tile_fft_ct_cols<R, N, EPT, false, W, T, true>(sm, s_tw, gload, mstore);
     auto sload = [&](int l, int a) -> Cx { return sm[a * W + l]; };
-    tile_fft_ct_cols<R, N, EPT, true, W, T>(sm, s_tw, sload, gstore);
+    tile_fft_ct_cols<R, N, EPT, true, W, T, true>(sm, s_tw, sload, gstore);
   }
 }
 
@@ -838,7 +838,7 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, DGPE_MINB_FFT_F32) k_fft_stride
 // table: four bytes less per spectrum element and no global load inside the
 // transform pair.
 template <int EPT, int MODE, int N, int W, int AXIS>
-__global__ void __launch_bounds__(DGPE_MAXT_FFT, DGPE_TMA_MINB)
+__global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
     k_fft_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ SArgs<float> A, int ncb, int ntiles,
               double *timeout_flag) {
   typedef float R;
@@ -891,9 +891,9 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, DGPE_TMA_MINB)
     auto sload = [&](int l, int a) -> Cx { return sm[a * W + l]; };
     auto sstore = [&](int l, int a, Cx v) { sm[a * W + l] = v; };
     if constexpr (MODE == 0) {
-      tile_fft_ct_cols<R, N, EPT, false, W, T>(sm, s_tw, sload, sstore);
+      tile_fft_ct_cols<R, N, EPT, false, W, T, true>(sm, s_tw, sload, sstore);
     } else if constexpr (MODE == 1) {
-      tile_fft_ct_cols<R, N, EPT, true, W, T>(sm, s_tw, sload, sstore);
+      tile_fft_ct_cols<R, N, EPT, true, W, T, true>(sm, s_tw, sload, sstore);
     } else if constexpr (AXIS == 2) {
       // tile: kx = c0 + l, ky = o, kz = row a
       const int jy = (o <= A.uny / 2) ? o : o - A.uny;
@@ -905,8 +905,8 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, DGPE_TMA_MINB)
         const R u = (k2 > (R)0) ? pref * ((R)3 * qz2 / k2 - (R)1) : (R)0;
         sm[a * W + l] = cscale(v, u);
       };
-      tile_fft_ct_cols<R, N, EPT, false, W, T>(sm, s_tw, sload, mstore);
-      tile_fft_ct_cols<R, N, EPT, true, W, T>(sm, s_tw, sload, sstore);
+      tile_fft_ct_cols<R, N, EPT, false, W, T, true>(sm, s_tw, sload, mstore);
+      tile_fft_ct_cols<R, N, EPT, true, W, T, true>(sm, s_tw, sload, sstore);
     } else {
       const size_t base = (size_t)o * A.ostride + c0;
       const long long es = A.estride;
@@ -914,8 +914,8 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, DGPE_TMA_MINB)
         const R u = (c0 + l < A.ncols) ? A.U[base + a * es + l] : (R)0;
         sm[a * W + l] = cscale(v, u);
       };
-      tile_fft_ct_cols<R, N, EPT, false, W, T>(sm, s_tw, sload, mstore);
-      tile_fft_ct_cols<R, N, EPT, true, W, T>(sm, s_tw, sload, sstore);
+      tile_fft_ct_cols<R, N, EPT, false, W, T, true>(sm, s_tw, sload, mstore);
+      tile_fft_ct_cols<R, N, EPT, true, W, T, true>(sm, s_tw, sload, sstore);
     }
     // the transformed tile goes back by tensor-map stores
     fence_proxy_async_smem();
