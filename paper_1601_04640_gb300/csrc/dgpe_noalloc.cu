@@ -43,37 +43,33 @@ size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // Roots w[t] = exp(-2 pi i t / n) per axis, U(k)/N on the half spectrum
 // [z][y][kx] (pitch px), and the parameter block (sc = 1, everything else 0).
+// FP64 work at 64 cycles per warp instruction and scheduler is what this costs:
+// U depends on |ky| and |kz| alone, so each value is computed once and written
+// to its two (2D) or four (3D) places, from wavenumber steps dq = 2 pi / (n h)
+// and the factor 1 / N that the host forms; one division (3D) is left.
 template <typename R>
 __global__ void k_noalloc_tables(cx<R> *tw0, cx<R> *tw1, cx<R> *tw2, R *U, double *prm,
                                  long long *step, int dim, int nx, int ny, int nz, int px,
-                                 double hx, double hy, double hz, int kernel, double qd) {
-  const size_t gid = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  const size_t gs = (size_t)gridDim.x * blockDim.x;
+                                 double dqx, double dqy, double dqz, int kernel, double qd, double pref, double rN) {
+  const unsigned gid = blockIdx.x * blockDim.x + threadIdx.x, gs = gridDim.x * blockDim.x;
   const int ns[3] = {nx, ny, nz};
   cx<R> *tw[3] = {tw0, tw1, tw2};
   for (int a = 0; a < dim; ++a)
-    for (size_t t = gid; t < (size_t)ns[a]; t += gs) {
+    for (unsigned t = gs - 1 - gid; t < (unsigned)ns[a]; t += gs) {  // the threads with the fewest U values
       double s, c;
       sincospi(-2.0 * (double)t / (double)ns[a], &s, &c);
       tw[a][t] = mk<R>((R)c, (R)s);
     }
-  const int nxh = nx / 2 + 1;
-  const size_t nspec = (size_t)nxh * ny * nz;
-  const double N = (double)nx * ny * nz;
-  const double twopi = 6.283185307179586476925286766559;
-  for (size_t i = gid; i < nspec; i += gs) {
-    const int kx = (int)(i % nxh);
-    const size_t r = i / nxh;
-    const int ky = (int)(r % ny), kz = (int)(r / ny);
-    const double qx = twopi * (double)(kx <= nx / 2 ? kx : kx - nx) / (nx * hx);
-    const double qy = twopi * (double)(ky <= ny / 2 ? ky : ky - ny) / (ny * hy);
+  const unsigned nxh = nx / 2 + 1, nyh = ny / 2 + 1, nzh = nz / 2 + 1, cnt = nxh * nyh * nzh;
+  for (unsigned i = gid; i < cnt; i += gs) {
+    const unsigned kx = i % nxh, r = i / nxh, ky = r % nyh, kz = r / nyh;
+    const double qx = (double)kx * dqx, qy = (double)ky * dqy;
     double u = 0.0;
     if (kernel == DGPE_KERNEL_DIPOLAR_3D) {
-      const double qz = twopi * (double)(kz <= nz / 2 ? kz : kz - nz) / (nz * hz);
-      const double k2 = qx * qx + qy * qy + qz * qz;
-      u = (k2 == 0.0) ? 0.0 : (4.0 * M_PI / 3.0) * (3.0 * qz * qz / k2 - 1.0);
+      const double qz = (double)kz * dqz, z2 = qz * qz, k2 = fma(qx, qx, fma(qy, qy, z2));
+      u = (k2 == 0.0) ? 0.0 : pref * fma(3.0, z2 / k2, -1.0);
     } else if (kernel == DGPE_KERNEL_QUASI2D_XY) {
-      const double q = sqrt(qx * qx + qy * qy) * qd, v = q / sqrt(2.0);
+      const double q = sqrt(qx * qx + qy * qy) * qd, v = q * 0.70710678118654752440;
       double ex;
       if (v < 25.0) {
         ex = exp(v * v) * erfc(v);
@@ -82,9 +78,14 @@ __global__ void k_noalloc_tables(cx<R> *tw0, cx<R> *tw1, cx<R> *tw2, R *U, doubl
         for (int m = 1; m < 8; ++m) { term *= -(2.0 * m - 1.0) / (2.0 * v * v); sum += term; }
         ex = sum / (v * sqrt(M_PI));
       }
-      u = (4.0 * M_PI / 3.0) / (sqrt(2.0 * M_PI) * qd) * (2.0 - 3.0 * sqrt(M_PI / 2.0) * q * ex);
+      u = pref * (2.0 - 3.0 * sqrt(M_PI / 2.0) * q * ex);
     }
-    U[r * px + kx] = (R)(u / N);
+    const R ur = (R)(u * rN);
+    const unsigned my = ky ? ny - ky : 0, mz = kz ? nz - kz : 0;
+    U[((size_t)kz * ny + ky) * px + kx] = ur;
+    U[((size_t)kz * ny + my) * px + kx] = ur;
+    U[((size_t)mz * ny + ky) * px + kx] = ur;
+    U[((size_t)mz * ny + my) * px + kx] = ur;
   }
   if (gid < PRM_COUNT) prm[gid] = (gid == PRM_SC) ? 1.0 : 0.0;
   if (gid == 0) *step = 0;
@@ -149,8 +150,14 @@ int run(const void *psi, void *phi, int dim, const int *n, const double *h, int 
     set_err("cudaFuncSetAttribute", cudaGetErrorString(e));
     return DGPE_ECUDA;
   }
-  k_noalloc_tables<R><<<64, 256, 0, s>>>(tw[0], tw[1], tw[2], U, prm, step, dim, nx, ny, nz, px,
-                                          h[0], h[1], dim == 3 ? h[2] : 1.0, kernel, qd);
+  {
+    const double twopi = 6.283185307179586476925286766559, hz = dim == 3 ? h[2] : 1.0;
+    const double pref = kernel == DGPE_KERNEL_DIPOLAR_3D ? 4.0 * M_PI / 3.0 : (4.0 * M_PI / 3.0) / (sqrt(2.0 * M_PI) * qd);
+    const int cnt = (nx / 2 + 1) * (ny / 2 + 1) * (nz / 2 + 1);
+    k_noalloc_tables<R><<<std::min((cnt + 63) / 64, 152 * 8), 64, 0, s>>>(
+        tw[0], tw[1], tw[2], U, prm, step, dim, nx, ny, nz, px, twopi / (nx * h[0]), twopi / (ny * h[1]), twopi / (nz * hz),
+        kernel, qd, pref, 1.0 / ((double)nx * ny * nz));
+  }
   XArgs<R> X{};
   X.psi = (Cx *)psi; X.spec = spec; X.phi_out = (R *)phi; X.prm = prm; X.step = step;
   X.tw = tw[0]; X.pl = plx; X.nx = nx; X.ny = ny; X.nrows = nrows; X.px = px; X.LP = LP;
