@@ -134,10 +134,9 @@ template <typename R> __device__ __forceinline__ void sin_cosm1(R x, R *sn, R *c
     *sn = x + (x * x2) * ps;
     *cm1 = x2 * pc;
   } else {
-    R s, c;
-    fsincos(x * (R)0.5, &s, &c);
-    *cm1 = (R)-2 * s * s;
-    *sn = (R)2 * s * c;
+    const cx<R> e = sincos_call(x * (R)0.5);
+    *cm1 = (R)-2 * e.x * e.x;
+    *sn = (R)2 * e.x * e.y;
   }
 }
 
