@@ -8,9 +8,17 @@
 namespace dgpe {
 namespace {
 
-// Columns per block of 256 threads: 8 (32 chunks) to 128 (2 chunks).
+// Columns per block of 256 threads: 8 (32 chunks) to 128 (2 chunks), halved
+// while a grid leaves SMs without a block, to blocks of one warp or segments of
+// two columns.
 constexpr int kColsThreads = 256;
-inline int cols_width(int n, int cl) { return kColsThreads / (n / cl); }
+inline int cols_lw(int n, int cl, unsigned tot, int nsm) {
+  const int tpl = n / cl;
+  int lw = 0;
+  while ((2 << lw) * tpl <= kColsThreads) ++lw;
+  while (lw > 1 && (1 << lw) * tpl > 32 && (tot >> lw) < (unsigned)nsm) --lw;
+  return lw;
+}
 
 // One thread holds CL consecutive points of one column in registers; the n /
 // CL chunks of a column are threads of the same block, and a warp is 32 (8,
@@ -37,6 +45,7 @@ __global__ void __launch_bounds__(kColsThreads, 3)
   float2 *const se = reinterpret_cast<float2 *>(smraw);  // chunk ends: forward, backward
   Coef *const tm = reinterpret_cast<Coef *>(se + 2 * T);  // TAB: -2 kt m, alpha, P, Q
   const Coef *const ta = tm + n, *const tp = ta + n, *const tq = tp + n;
+  pdl_wait();
   if (TAB) {
     const Coef *g = reinterpret_cast<const Coef *>(A.cntab);
     const Coef m2kt = coef_scale(make_kt<Coef>(A.tau), -2.0f);
@@ -63,31 +72,7 @@ __global__ void __launch_bounds__(kColsThreads, 3)
       if (q < tpl - 1) next = p[(size_t)CL * A.es];
     }
     if constexpr (!TAB) {
-      se[t] = cn_chunk_forward<Coef, CL>(v, prev, next, K, y);
-      __syncthreads();
-      float2 in = make_float2(0.0f, 0.0f);
-      for (int j = max(0, q - K.dl); j < q; ++j) in = coef_fma(K.pc, in, se[(j << lw) + lc]);
-      float2 *const sb = se + T;
-      sb[t] = cn_chunk_backward<Coef, CL>(in, K, y);
-      __syncthreads();
-      in = make_float2(0.0f, 0.0f);
-      for (int j = min(tpl - 1, q + K.dl); j > q; --j) in = coef_fma(K.pc, in, sb[(j << lw) + lc]);
-      cn_chunk_inflow<Coef, CL>(in, K, y);
-      // u_0 of the column is the first chunk's y[0]
-      float2 img = make_float2(0.0f, 0.0f);
-      if (K.dl == 1) {
-        if (q == 0) img = coef_mul(K.al, y[0]);
-      } else {
-        __syncthreads();  // the forward ends have been read
-        if (q == 0) se[lc] = y[0];
-        __syncthreads();
-        if (q < K.dl) {
-          img = coef_mul(K.al, se[lc]);
-          for (int j = 0; j < q; ++j) img = coef_mul(K.pc, img);
-        }
-        __syncthreads();  // before the next tile's forward ends
-      }
-      cn_chunk_finish<Coef, CL>(img, K, y, v);
+      col_solve<Coef, CL>(v, y, prev, next, q, tpl, lw, lc, se, K);
     } else {
       float2 e = make_float2(0.0f, 0.0f);
 #pragma unroll
@@ -168,11 +153,6 @@ template <class F> cudaError_t with_chunk(int cl, F &&f) {
   }
 }
 
-inline int cols_lw(int n, int cl) {
-  int lw = 0;
-  while ((1 << lw) < cols_width(n, cl)) ++lw;
-  return lw;
-}
 template <typename Coef> size_t cols_smem(int n, int T, bool tab) {
   return sizeof(float2) * 2 * (size_t)T + (tab ? sizeof(Coef) * 4 * (size_t)n : 0);
 }
@@ -188,7 +168,7 @@ template <typename Coef, class F> cudaError_t with_kernel(int cl, bool norm, boo
   });
 }
 template <typename Coef> int grid_of(int n, int cl, unsigned tot, int nsm, bool tab) {
-  const int w = cols_width(n, cl), T = w * (n / cl), ntiles = (int)((tot + (unsigned)w - 1) / (unsigned)w);
+  const int w = 1 << cols_lw(n, cl, tot, nsm), T = w * (n / cl), ntiles = (int)((tot + (unsigned)w - 1) / (unsigned)w);
   int occ = 0;
   with_kernel<Coef>(cl, true, tab, [&](auto k) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, T, cols_smem<Coef>(n, T, tab));
@@ -196,12 +176,11 @@ template <typename Coef> int grid_of(int n, int cl, unsigned tot, int nsm, bool 
   return std::max(1, std::min(ntiles, nsm * std::max(occ, 1)));
 }
 template <typename Coef> cudaError_t launch(const ColArgs &A, const CnConst<Coef> &K, int grid, cudaStream_t s) {
-  const int w = cols_width(A.n, A.cl), T = w * (A.n / A.cl), lw = cols_lw(A.n, A.cl);
+  const int lw = cols_lw(A.n, A.cl, A.tot, A.nsm), w = 1 << lw, T = w * (A.n / A.cl);
   const int ntiles = (int)((A.tot + (unsigned)w - 1) / (unsigned)w);
   const bool tab = K.dl == 0;
   return with_kernel<Coef>(A.cl, A.norm != 0, tab, [&](auto k) {
-    k<<<grid, T, cols_smem<Coef>(A.n, T, tab), s>>>(A, K, lw, ntiles);
-    return cudaGetLastError();
+    return launch_pdl(A.early != 0, k, dim3(grid), T, cols_smem<Coef>(A.n, T, tab), s, A, K, lw, ntiles);
   });
 }
 

@@ -584,6 +584,17 @@ __device__ __forceinline__ void tile_fft_ct_cols(cx<R> *sm, const cx<R> *__restr
   tile_fft_ct_from<R, N, EPT, INV, 0, 1, NL, T, true, NL, 0, 1, PF>(sm, tw, load, store);
 }
 
+// ------------------------------------------------ programmatic launch order
+// The passes of a step are launched so that a pass's blocks start while the
+// one before it drains (launch_pdl): they set up what only constants need and
+// wait here until that pass has completed and its writes are visible.  Every
+// pass waits before its first access to anything a pass writes, so completion
+// stays in order over any number of passes.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
 // ------------------------------------------- Crank-Nicolson (Thomas) solve
 // One CN substep along a line of n points, in increment form:
 //   x = psi + w,  A w = r,  r = -2 kt (2 psi_a - psi_{a-1} - psi_{a+1}),

@@ -197,6 +197,12 @@ template <class F> int with_pow2_len(int n, F &&f) {
   }
 }
 
+// largest grid whose passes start while the one before drains (128^3 FP32: 51
+// us a step without, 59 with it; 64^3: 30.8 and 28.6 us)
+constexpr size_t kEarlySites = (size_t)1 << 18;
+// largest grid with a graph of several steps: above it a step takes some 100 us,
+// beside which the gap between two graphs is small
+constexpr size_t kRunSites = (size_t)1 << 22;
 // Call f(N, EPT) for any line length of the FP32 strided transforms (EPT
 // elements per thread: 16, 12 or 20 for 2^k, 3 2^k, 5 2^k).
 template <class F> int with_col_len(int n, F &&f) {
@@ -298,8 +304,12 @@ template <typename R> struct EngineT : Engine {
   int obs_rows = 1, obs_blocks = 0, ndip = 0;
 
   cudaStream_t cap = nullptr;
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t gexec = nullptr;
+  // one step, and (small grids) kRunSteps of them: between the steps of one
+  // graph a pass starts while the one before it drains, between two graphs the
+  // GPU idles
+  static constexpr int kRunSteps = 4;
+  bool early = false;
+  cudaGraphExec_t gexec = nullptr, grun = nullptr;
   bool use_graph = true;
   bool strang = false;  // second-order splitting (real time)
   // real state (imaginary time): psi holds nx reals per row, viewed by the
@@ -309,7 +319,7 @@ template <typename R> struct EngineT : Engine {
 
   ~EngineT() override {
     if (gexec) cudaGraphExecDestroy(gexec);
-    if (graph) cudaGraphDestroy(graph);
+    if (grun) cudaGraphExecDestroy(grun);
     if (cap) cudaStreamDestroy(cap);
     void *bufs[] = {psi, spec, U, phi_tmp, tw[0], tw[1], tw[2], vt[0], vt[1], vt[2],
                     cntab[0], cntab[1], cntab[2], prm, partial, obs_part, dip_part, obs_out,
@@ -362,6 +372,12 @@ template <typename R> struct EngineT : Engine {
 
     // kernel variants and FFT plans
     const int nsz[3] = {nx, ny, nz};
+    {
+      int dev = 0;
+      DGPE_CK(cudaGetDevice(&dev));
+      DGPE_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    }
+    early = nsites <= kEarlySites;
     for (int a = 0; a < dim; ++a) {
       var[a] = axis_variant(nsz[a]);
       if (var[a] == VAR_NONE) {
@@ -465,13 +481,19 @@ template <typename R> struct EngineT : Engine {
         while (w > 1 && w * n / ept > DGPE_MAXT_FFT) w >>= 1;
         return w;
       };
-      const int ey = variant_ept_s(var[1], EPT_S);
-      fy.n = ny; fy.W = wfor(ny, ey); fy.T = fy.W * ny / ey; fy.es = px; fy.os = (long long)ny * px;
-      fy.grid = dim3((ncol_spec + fy.W - 1) / fy.W, nz); fy.smem = sizeof(Cx) * (size_t)ny * fy.W; fy.pl = ply;
+      auto config = [&](FtCfg &f, int axis, int n, int outer) {
+        const int e = variant_ept_s(var[axis], EPT_S);
+        f.n = n;
+        f.W = wfor(n, e);
+        f.T = f.W * n / e;
+        f.grid = dim3((ncol_spec + f.W - 1) / f.W, outer);
+        f.smem = sizeof(Cx) * (size_t)n * f.W;
+      };
+      config(fy, 1, ny, nz);
+      fy.es = px; fy.os = (long long)ny * px; fy.pl = ply;
       if (dim == 3) {
-        const int ez = variant_ept_s(var[2], EPT_S);
-        fz.n = nz; fz.W = wfor(nz, ez); fz.T = fz.W * nz / ez; fz.es = (long long)ny * px; fz.os = px;
-        fz.grid = dim3((ncol_spec + fz.W - 1) / fz.W, ny); fz.smem = sizeof(Cx) * (size_t)nz * fz.W; fz.pl = plz;
+        config(fz, 2, nz, ny);
+        fz.es = (long long)ny * px; fz.os = px; fz.pl = plz;
       }
       if (fy.T > DGPE_MAXT_FFT || fz.T > DGPE_MAXT_FFT) { err = "strided FFT block too large"; return DGPE_EUNSUPPORTED; }
     }
@@ -482,9 +504,10 @@ template <typename R> struct EngineT : Engine {
     const CnCfg &fin = cn[dim == 3 ? 2 : 1];
     const LnCfg &lfin = ln[dim == 3 ? 2 : 1];
     // norm partials of the final pass (twice its default grid: a batch may run
-    // the pass with half-width tiles)
-    if ((rc = dalloc(&partial, std::max(2 * (size_t)fin.grid.x * fin.grid.y,
-                                        cn_serial ? (size_t)lfin.grid.x * lfin.grid.y : (size_t)0)))) return rc;
+    // the pass with half-width tiles; the FP32 pass narrows its tiles to at
+    // most 2 nsm of them)
+    if ((rc = dalloc(&partial, std::max({2 * (size_t)fin.grid.x * fin.grid.y, 2 * (size_t)nsm + 2,
+                                         cn_serial ? (size_t)lfin.grid.x * lfin.grid.y : (size_t)0})))) return rc;
     if ((rc = dalloc(&obs_part, (size_t)obs_blocks * OBS_COUNT))) return rc;
     if ((rc = dalloc(&dip_part, (size_t)std::max(ndip, 1)))) return rc;
     if ((rc = dalloc(&obs_out, OBS_COUNT + 1))) return rc;
@@ -713,11 +736,6 @@ template <typename R> struct EngineT : Engine {
     return DGPE_OK;
   }
   int set_smem_attrs() {
-    {
-      int dev = 0;
-      DGPE_CK(cudaGetDevice(&dev));
-      DGPE_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    }
     int rc = with_xvar(var[0], [&](auto CLc, auto EXc, auto P2c) -> int {
       constexpr int CL = decltype(CLc)::value, EX = decltype(EXc)::value;
       constexpr bool P2 = decltype(P2c)::value;
@@ -872,16 +890,28 @@ template <typename R> struct EngineT : Engine {
       if (mode > 2) return false;
       bool done = false;
       with_col_len(f.n, [&](auto Nc, auto Ec) -> int {
-        constexpr int N = decltype(Nc)::value, E = decltype(Ec)::value, WW = col_width(N, E);
+        constexpr int N = decltype(Nc)::value, E = decltype(Ec)::value, WW = col_width(N, E), WN = narrow_width(N, E);
         if (f.W != WW) return 0;
-        if (mode == 0) k_fft_strided_ct<E, 0, N, WW><<<f.grid, f.T, f.smem, s>>>(A);
-        else if (mode == 1) k_fft_strided_ct<E, 1, N, WW><<<f.grid, f.T, f.smem, s>>>(A);
-        else k_fft_strided_ct<E, 2, N, WW><<<f.grid, f.T, f.smem, s>>>(A);
+        if (narrow(f, mode)) {
+          launch_pdl(early, k_fft_strided_ct<E, 2, N, WN>, dim3((ncol_spec + WN - 1) / WN), WN * N / E,
+                     sizeof(Cx) * (size_t)WN * N, s, A);
+          done = true;
+          return 0;
+        }
+        if (mode == 0) launch_pdl(early, k_fft_strided_ct<E, 0, N, WW>, f.grid, f.T, f.smem, s, A);
+        else if (mode == 1) launch_pdl(early, k_fft_strided_ct<E, 1, N, WW>, f.grid, f.T, f.smem, s, A);
+        else launch_pdl(early, k_fft_strided_ct<E, 2, N, WW>, f.grid, f.T, f.smem, s, A);
         done = true;
         return 0;
       });
       return done;
     }
+  }
+  // A plane's one strided pass has few tiles (9 of 16 columns at 256^2): tiles
+  // of one warp, or of two columns, where they spread over more SMs.
+  static constexpr int narrow_width(int n, int ept) { return 32 * ept / n > 2 ? 32 * ept / n : 2; }
+  bool narrow(const FtCfg &f, int mode) const {
+    return !(p.flags & DGPE_FLAG_P1_ONESHOT) && dim == 2 && mode == 2 && (int)f.grid.x < nsm;
   }
   // Tile width of a strided FP32 transform: DGPE_W_FFT_F32 columns, halved
   // until a block has at most DGPE_MAXT_FFT threads.
@@ -951,17 +981,17 @@ template <typename R> struct EngineT : Engine {
     if constexpr (sizeof(R) != 4) {
       return false;
     } else {
-      if (!tma_fft || mode > 2 || (f.axis == 2 && mode != 2)) return false;
+      if (!tma_fft || mode > 2 || (f.axis == 2 && mode != 2) || narrow(f, mode)) return false;
       const int ncb = (int)f.grid.x, ntiles = (int)(f.grid.x * f.grid.y);
       const int g = std::max(1, std::min(ntiles, tma_grid[f.axis - 1]));
       double *tf = prm + PRM_TIMEOUT;
       with_col_len(f.n, [&](auto Nc, auto Ec) -> int {
         constexpr int N = decltype(Nc)::value, E = decltype(Ec)::value, WW = col_width(N, E), T = WW * N / E;
         const size_t sm = 2 * sizeof(Cx) * (size_t)WW * N + 128;
-        if (f.axis == 2) k_fft_tma<E, 2, N, WW, 2><<<g, T, sm, s>>>(tm_z, A, ncb, ntiles, tf);
-        else if (mode == 0) k_fft_tma<E, 0, N, WW, 1><<<g, T, sm, s>>>(tm_y, A, ncb, ntiles, tf);
-        else if (mode == 1) k_fft_tma<E, 1, N, WW, 1><<<g, T, sm, s>>>(tm_y, A, ncb, ntiles, tf);
-        else k_fft_tma<E, 2, N, WW, 1><<<g, T, sm, s>>>(tm_y, A, ncb, ntiles, tf);
+        if (f.axis == 2) launch_pdl(early, k_fft_tma<E, 2, N, WW, 2>, dim3(g), T, sm, s, tm_z, A, ncb, ntiles, tf);
+        else if (mode == 0) launch_pdl(early, k_fft_tma<E, 0, N, WW, 1>, dim3(g), T, sm, s, tm_y, A, ncb, ntiles, tf);
+        else if (mode == 1) launch_pdl(early, k_fft_tma<E, 1, N, WW, 1>, dim3(g), T, sm, s, tm_y, A, ncb, ntiles, tf);
+        else launch_pdl(early, k_fft_tma<E, 2, N, WW, 1>, dim3(g), T, sm, s, tm_y, A, ncb, ntiles, tf);
         return 0;
       });
       return true;
@@ -980,10 +1010,10 @@ template <typename R> struct EngineT : Engine {
       constexpr bool FM = P2 && (sizeof(R) == 8 || DGPE_FFT_FMA_F32);  // FMA-form twiddled stages
       constexpr bool FM1 = P2 && sizeof(R) == 8;  // the C2R pass: FP64 only
       switch (mode) {
-        case 0: k_fft_strided<R, EP, 0, P2, FM><<<f.grid, f.T, f.smem, s>>>(A); break;
-        case 1: k_fft_strided<R, EP, 1, P2, FM><<<f.grid, f.T, f.smem, s>>>(A); break;
-        case 2: k_fft_strided<R, EP, 2, P2, FM><<<f.grid, f.T, f.smem, s>>>(A); break;
-        default: k_fft_strided<R, EP, 3, P2, FM><<<f.grid, f.T, f.smem, s>>>(A); break;
+        case 0: launch_pdl(early, k_fft_strided<R, EP, 0, P2, FM>, f.grid, f.T, f.smem, s, A); break;
+        case 1: launch_pdl(early, k_fft_strided<R, EP, 1, P2, FM>, f.grid, f.T, f.smem, s, A); break;
+        case 2: launch_pdl(early, k_fft_strided<R, EP, 2, P2, FM>, f.grid, f.T, f.smem, s, A); break;
+        default: launch_pdl(early, k_fft_strided<R, EP, 3, P2, FM>, f.grid, f.T, f.smem, s, A); break;
       }
       return DGPE_OK;
     });
@@ -1000,8 +1030,8 @@ template <typename R> struct EngineT : Engine {
       A.cntab = adjoint ? cntab_adj[axis] : cntab[axis];
       A.prm = prm; A.partial = partial; A.counter = counter; A.step = dstep;
       A.es = c.es; A.os = c.os; A.ncols = (unsigned)c.ncols; A.tot = (unsigned)c.ncols * c.grid.y;
-      A.n = c.n; A.cl = c.C; A.final_pass = final_pass ? 1 : 0; A.norm = (final_pass && imag) ? 1 : 0;
-      A.dlim = cn_dlim[axis]; A.tau = adjoint ? -tau[axis] : tau[axis];
+      A.n = c.n; A.cl = c.C; A.nsm = nsm; A.final_pass = final_pass ? 1 : 0; A.norm = (final_pass && imag) ? 1 : 0;
+      A.early = early ? 1 : 0; A.dlim = cn_dlim[axis]; A.tau = adjoint ? -tau[axis] : tau[axis];
       const cudaError_t e = imag ? cols_launch(A, cn_kr[axis], cols_pgrid[axis], s)
                                  : cols_launch(A, adjoint ? cn_ka[axis] : cn_kc[axis], cols_pgrid[axis], s);
       launched(1);
@@ -1018,7 +1048,7 @@ template <typename R> struct EngineT : Engine {
     if constexpr (sizeof(R) == 4) {
       A.psi = psi; A.spec = spec; A.phi_out = phi_tmp; A.prm = prm; A.step = dstep;
       A.tw = tw[0]; A.vx = vt[0]; A.vy = vt[1]; A.vz = vt[2];
-      A.n = nx; A.ny = ny; A.nrows = nrows; A.has_dip = has_dip ? 1 : 0; A.dtf = 1.0;
+      A.n = nx; A.ny = ny; A.nrows = nrows; A.has_dip = has_dip ? 1 : 0; A.dtf = 1.0; A.early = early ? 1 : 0;
     }
     return A;
   }
@@ -1078,9 +1108,9 @@ template <typename R> struct EngineT : Engine {
     with_cl(var[axis], [&](auto CLc) -> int {
       constexpr int CL = decltype(CLc)::value;
       // the norm's code only in the pass that takes the norm
-      if (imag && A.norm) k_cn_strided_pipe<R, R, CL, true><<<c.pgrid[0], c.T, 2 * c.smem, s>>>(A, ncb, ntiles);
-      else if (imag) k_cn_strided_pipe<R, R, CL, false><<<c.pgrid[0], c.T, 2 * c.smem, s>>>(A, ncb, ntiles);
-      else k_cn_strided_pipe<R, Cx, CL, false><<<c.pgrid[1], c.T, 2 * c.smem, s>>>(A, ncb, ntiles);
+      if (imag && A.norm) launch_pdl(early, k_cn_strided_pipe<R, R, CL, true>, dim3(c.pgrid[0]), c.T, 2 * c.smem, s, A, ncb, ntiles);
+      else if (imag) launch_pdl(early, k_cn_strided_pipe<R, R, CL, false>, dim3(c.pgrid[0]), c.T, 2 * c.smem, s, A, ncb, ntiles);
+      else launch_pdl(early, k_cn_strided_pipe<R, Cx, CL, false>, dim3(c.pgrid[1]), c.T, 2 * c.smem, s, A, ncb, ntiles);
       return DGPE_OK;
     });
     launched(1);
@@ -1095,9 +1125,9 @@ template <typename R> struct EngineT : Engine {
     A.es = L.es; A.cs = L.cs; A.os = L.os; A.n = L.n; A.ncols = L.ncols;
     A.final_pass = final_pass ? 1 : 0; A.norm = (final_pass && imag) ? 1 : 0;
     A.tau = adjoint ? -tau[axis] : tau[axis];
-    if (imag && A.norm) k_cn_lines<R, R, true><<<L.grid, L.T, 0, s>>>(A);
-    else if (imag) k_cn_lines<R, R, false><<<L.grid, L.T, 0, s>>>(A);
-    else k_cn_lines<R, Cx, false><<<L.grid, L.T, 0, s>>>(A);
+    if (imag && A.norm) launch_pdl(early, k_cn_lines<R, R, true>, L.grid, L.T, 0, s, A);
+    else if (imag) launch_pdl(early, k_cn_lines<R, R, false>, L.grid, L.T, 0, s, A);
+    else launch_pdl(early, k_cn_lines<R, Cx, false>, L.grid, L.T, 0, s, A);
     launched(1);
     DGPE_LCK(__func__);
     return DGPE_OK;
@@ -1118,9 +1148,9 @@ template <typename R> struct EngineT : Engine {
       constexpr bool P2 = decltype(P2c)::value;
       constexpr bool FM = P2 && (sizeof(R) == 8 || DGPE_FFT_FMA_F32);  // FMA-form twiddled stages
       constexpr bool FM1 = P2 && sizeof(R) == 8;  // the C2R pass: FP64 only
-      if (dens_in) k_dens_r2c_x<R, EX, 1, P2, FM><<<x_grid, x_T, x4_smem, s>>>(A);
-      else if (rpsi && !src) k_dens_r2c_x<R, EX, 2, P2, FM><<<x_grid, x_T, x4_smem, s>>>(A);
-      else k_dens_r2c_x<R, EX, 0, P2, FM><<<x_grid, x_T, x4_smem, s>>>(A);
+      if (dens_in) launch_pdl(early, k_dens_r2c_x<R, EX, 1, P2, FM>, dim3(x_grid), x_T, x4_smem, s, A);
+      else if (rpsi && !src) launch_pdl(early, k_dens_r2c_x<R, EX, 2, P2, FM>, dim3(x_grid), x_T, x4_smem, s, A);
+      else launch_pdl(early, k_dens_r2c_x<R, EX, 0, P2, FM>, dim3(x_grid), x_T, x4_smem, s, A);
       return DGPE_OK;
     });
     launched(1);
@@ -1153,27 +1183,27 @@ template <typename R> struct EngineT : Engine {
       constexpr bool FM = P2 && (sizeof(R) == 8 || DGPE_FFT_FMA_F32);  // FMA-form twiddled stages
       constexpr bool FM1 = P2 && sizeof(R) == 8;  // the C2R pass: FP64 only
       if (mode == 0 && rpsi) {
-        k_c2r_x_exp_cnx<R, R, EX, CL, 4, P2, FM1><<<x_grid, x_T, x_smem, s>>>(A);
+        launch_pdl(early, k_c2r_x_exp_cnx<R, R, EX, CL, 4, P2, FM1>, dim3(x_grid), x_T, x_smem, s, A);
       } else if (mode == 0 && p1_pipe) {
         if constexpr (sizeof(R) == 4 && P2 && CL == 16) {
           with_pow2_len(nx, [&](auto Nc) -> int {
             constexpr int N = decltype(Nc)::value;
             if constexpr (N != 0) {
-              if (imag) k_p1_pipe<R, EX, CL, N><<<p1_grid[0], x_T, p1_smem[0], s>>>(A, x_grid, nz, prm + PRM_TIMEOUT);
-              else k_p1_pipe<Cx, EX, CL, N><<<p1_grid[1], x_T, p1_smem[1], s>>>(A, x_grid, nz, prm + PRM_TIMEOUT);
+              if (imag) launch_pdl(early, k_p1_pipe<R, EX, CL, N>, dim3(p1_grid[0]), x_T, p1_smem[0], s, A, x_grid, nz, prm + PRM_TIMEOUT);
+              else launch_pdl(early, k_p1_pipe<Cx, EX, CL, N>, dim3(p1_grid[1]), x_T, p1_smem[1], s, A, x_grid, nz, prm + PRM_TIMEOUT);
             }
             return 0;
           });
         }
       } else if (mode == 0) {
-        if (imag) k_c2r_x_exp_cnx<R, R, EX, CL, 0, P2, FM1><<<x_grid, x_T, x_smem, s>>>(A);
-        else k_c2r_x_exp_cnx<R, Cx, EX, CL, 0, P2, FM1><<<x_grid, x_T, x_smem, s>>>(A);
+        if (imag) launch_pdl(early, k_c2r_x_exp_cnx<R, R, EX, CL, 0, P2, FM1>, dim3(x_grid), x_T, x_smem, s, A);
+        else launch_pdl(early, k_c2r_x_exp_cnx<R, Cx, EX, CL, 0, P2, FM1>, dim3(x_grid), x_T, x_smem, s, A);
       } else if (mode == 3) {
-        k_c2r_x_exp_cnx<R, R, EX, CL, 3, P2, FM1><<<x_grid, x_T, x_smem, s>>>(A);
+        launch_pdl(early, k_c2r_x_exp_cnx<R, R, EX, CL, 3, P2, FM1>, dim3(x_grid), x_T, x_smem, s, A);
       } else if (mode == 1) {
-        k_c2r_x_exp_cnx<R, R, EX, CL, 1, P2, FM1><<<x_grid, x_T, x_smem, s>>>(A);
+        launch_pdl(early, k_c2r_x_exp_cnx<R, R, EX, CL, 1, P2, FM1>, dim3(x_grid), x_T, x_smem, s, A);
       } else {
-        k_c2r_x_exp_cnx<R, Cx, EX, CL, 2, P2, FM1><<<x_grid, x_T, x_smem, s>>>(A);
+        launch_pdl(early, k_c2r_x_exp_cnx<R, Cx, EX, CL, 2, P2, FM1>, dim3(x_grid), x_T, x_smem, s, A);
       }
       return DGPE_OK;
     });
@@ -1364,20 +1394,27 @@ template <typename R> struct EngineT : Engine {
     for (int i = 0; i < np; ++i) pass_ms[i] = n > 0 ? acc[i] / n : 0.0;
     return np;
   }
-  int capture() {
-    if (gexec) { cudaGraphExecDestroy(gexec); gexec = nullptr; }
-    if (graph) { cudaGraphDestroy(graph); graph = nullptr; }
+  int capture(cudaGraphExec_t *exec, int n) {
+    if (*exec) { cudaGraphExecDestroy(*exec); *exec = nullptr; }
     DGPE_CK(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
     capturing = true;
-    int rc = launch_step(cap);
+    int rc = DGPE_OK;
+    for (int i = 0; i < n && !rc; ++i) rc = launch_step(cap);
     capturing = false;
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(cap, &g);
-    if (rc) { if (g) cudaGraphDestroy(g); return rc; }
-    if (e != cudaSuccess) { err = std::string("graph capture: ") + cudaGetErrorString(e); return DGPE_ECUDA; }
-    graph = g;
-    DGPE_CK(cudaGraphInstantiate(&gexec, graph, 0));
-    return DGPE_OK;
+    if (!rc && e != cudaSuccess) { err = std::string("graph capture: ") + cudaGetErrorString(e); rc = DGPE_ECUDA; }
+    if (!rc) {
+      e = cudaGraphInstantiate(exec, g, 0);
+      if (e != cudaSuccess) { err = std::string("graph instantiation: ") + cudaGetErrorString(e); rc = DGPE_ECUDA; }
+    }
+    if (g) cudaGraphDestroy(g);
+    return rc;
+  }
+  int capture() {
+    int rc = capture(&gexec, 1);
+    if (!rc && nsites <= kRunSites) rc = capture(&grun, kRunSteps);
+    return rc;
   }
 
   // ------------------------------------------------------------ API calls
@@ -1386,10 +1423,11 @@ template <typename R> struct EngineT : Engine {
     if (strang && n > 0 && (rc = launch_exp_only(-0.5, s))) return rc;
     for (int i = 0; i < n; ++i) {
       if (use_graph) {
-        DGPE_CK(cudaGraphLaunch(gexec, s));
-        nlaunch += launches_per_step();
-      }
-      else {
+        const bool run = grun && n - i >= kRunSteps;
+        DGPE_CK(cudaGraphLaunch(run ? grun : gexec, s));
+        nlaunch += (run ? kRunSteps : 1) * launches_per_step();
+        if (run) i += kRunSteps - 1;
+      } else {
         if ((rc = launch_step(s))) return rc;
       }
     }

@@ -265,9 +265,8 @@ __device__ __forceinline__ void dens_r2c_x_body(const XArgs<R> &A, int bx) {
   const int n = NC ? NC : A.nx, SL = NC ? SLC : A.pitchz, nrows = A.nrows, LP = NC ? LPC : A.LP;
   const int px = NC ? NC / 2 + 2 : A.px;
   const int p0 = bx * LP;
-  const R sc = (R)A.prm[PRM_SC];
-  const R sc2 = sc * sc;
   const cx<R> *__restrict__ psi = A.psi;
+  R sc2 = (R)1;
   auto load = [&](int l, int a) -> cx<R> {
     const int r0 = 2 * (p0 + l), r1 = r0 + 1;
     R d0 = 0, d1 = 0;
@@ -293,6 +292,9 @@ __device__ __forceinline__ void dens_r2c_x_body(const XArgs<R> &A, int bx) {
   rt4<R> *s_rt = reinterpret_cast<rt4<R> *>(scr + OFF_RT);
   const cx<R> *tw = FMA ? A.tw : stage_twiddles<R>(s_tw, A.tw, n);
   const rt4<R> *rt = FMA ? stage_roots(s_rt, A.twf, n) : nullptr;
+  if constexpr (SCR == 0) pdl_wait();
+  sc2 = (R)A.prm[PRM_SC];
+  sc2 *= sc2;
   if constexpr (NC > 0) tile_fft_ct<R, NC, EPT, false, PW, SLC, LPC, DGPE_MAXT>(zt, tw, load, store);
   else tile_fft<R, EPT, false, false, PW, POW2, FMA>(zt, SL, 1, A.LP, A.pl, tw, load, store, rt);
   // two real lines were packed as Z = n0 + i n1: X0 = (Z_k + conj Z_{n-k}) / 2,
@@ -386,6 +388,7 @@ __device__ __forceinline__ void c2r_x_exp_cnx_body(const XArgs<R> &A, int bx) {
   rt4<R> *const s_rt = reinterpret_cast<rt4<R> *>(scr + OFF_RT);
   const rt4<R> *rt = nullptr;
   if constexpr (FMA && MODE != 2) rt = stage_roots(s_rt, A.twi, n);
+  if constexpr (SCR == 0) pdl_wait();
   if constexpr (RS) {
     const R *__restrict__ pr = reinterpret_cast<const R *>(A.psi);
     R buf[CL];
@@ -614,6 +617,7 @@ __global__ void __launch_bounds__(DGPE_MAXT, 2) k_p1_pipe(const __grid_constant_
     bulk_g2s(sp, A.psi + (size_t)r0 * N, bp, &bar);
     if (dip) bulk_g2s(sz, A.spec + (size_t)r0 * PX, bs, &bar);
   };
+  pdl_wait();
   if (t == 0) {
     mbar_init(&bar, 1);
     s_k[0] = (R)(trap_dts(A.prm, *A.step) * A.dtf);
@@ -722,6 +726,7 @@ __device__ __forceinline__ void fft_strided_body(const SArgs<R> &A, int bx, int 
   const rt4<R> *rf = nullptr, *ri = nullptr;
   if constexpr (NF) rf = stage_roots(s_rf, A.twf, A.n);
   if constexpr (NI) ri = stage_roots(s_ri, A.twi, A.n);
+  if constexpr (SCR == 0) pdl_wait();
   const int W = NC ? WC : A.W;
   const int c0 = bx * W;
   const size_t base = (size_t)by * A.ostride + c0;
@@ -784,7 +789,8 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, DGPE_MINB_FFT(R, EPT)) k_fft_st
 // (power-of-two lengths): the same arithmetic as fft_strided_body, with every
 // index folded (tile_fft_ct_cols).  Twiddles from a shared copy.
 template <int EPT, int MODE, int N, int W>
-__global__ void __launch_bounds__(DGPE_MAXT_FFT, DGPE_MINB_FFT_F32) k_fft_strided_ct(const __grid_constant__ SArgs<float> A) {
+__global__ void __launch_bounds__(W * N / EPT < 128 ? 64 : DGPE_MAXT_FFT, W * N / EPT < 128 ? 8 : DGPE_MINB_FFT_F32)
+    k_fft_strided_ct(const __grid_constant__ SArgs<float> A) {
   typedef float R;
   typedef float2 Cx;
   constexpr int T = W * N / EPT;
@@ -792,6 +798,7 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, DGPE_MINB_FFT_F32) k_fft_stride
   Cx *sm = reinterpret_cast<Cx *>(smraw);  // [a][W]
   __shared__ __align__(16) Cx s_tw[N];
   for (int i = threadIdx.x; i < N; i += T) s_tw[i] = A.tw[i];
+  pdl_wait();
   __syncthreads();
   const int c0 = blockIdx.x * W;
   const size_t base = (size_t)blockIdx.y * A.ostride + c0;
@@ -865,13 +872,13 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
   }
+  for (int i = t; i < N; i += T) s_tw[i] = A.tw[i];
+  pdl_wait();
   __syncthreads();
   if (t == 0) {
     if ((int)blockIdx.x < ntiles) issue(blockIdx.x, 0);
     if ((int)(blockIdx.x + gridDim.x) < ntiles) issue(blockIdx.x + gridDim.x, 1);
   }
-  for (int i = t; i < N; i += T) s_tw[i] = A.tw[i];
-  __syncthreads();
   unsigned ph = 0u;  // bit k: the phase parity buffer k waits for next
   int k = 0;
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, k ^= 1) {
@@ -1068,6 +1075,7 @@ __global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB_CN(R)) k_cn_strided_pipe(
   constexpr bool TAB = (sizeof(R) == 8);
   __shared__ __align__(16) Coef s_tab[TAB ? 1 : 4 * (512 + 512 / CL + 1)];
   if (!TAB) stage_cn_tables<Coef, CL>(s_tab, reinterpret_cast<const Coef *>(A.cntab), n);  // visible after the loop's first barrier
+  pdl_wait();
   double acc = 0.0;
   int k = 0;
   if ((int)blockIdx.x < ntiles) fetch(blockIdx.x, buf[0]);
@@ -1222,6 +1230,7 @@ __global__ void __launch_bounds__(128) k_cn_lines(const __grid_constant__ LArgs 
   const R tau = (R)A.tau;
   const R one_m2tau = (sizeof(Coef) == sizeof(R)) ? (R)(1.0 - 2.0 * A.tau) : (R)(2.0 * A.tau);
   const Coef *tm = reinterpret_cast<const Coef *>(A.tab), *ta = tm + n;
+  pdl_wait();
   double acc = 0.0;
   if (c < A.ncols) {
     Cx *p = reinterpret_cast<Cx *>(A.psi) + (size_t)blockIdx.y * A.os + (size_t)c * A.cs;

@@ -86,5 +86,39 @@ __device__ __forceinline__ void cn_chunk_finish(float2 img, const CnConst<Coef> 
   for (int i = 0; i < CL; ++i) v[i] = v[i] + coef_mul(K.m2, y[i]);
 }
 
+
+// Solve of strided columns by a block: thread t holds chunk q = t >> lw of
+// column lc, the chunks exchange their ends through se (2 blockDim.x elements).
+template <typename Coef, int CL>
+__device__ __forceinline__ void col_solve(float2 (&v)[CL], float2 (&y)[CL], float2 prev, float2 next, int q, int tpl, int lw,
+                                          int lc, float2 *se, const CnConst<Coef> &K) {
+  const int t = threadIdx.x;
+  se[t] = cn_chunk_forward<Coef, CL>(v, prev, next, K, y);
+  __syncthreads();
+  float2 in = make_float2(0.0f, 0.0f);
+  for (int j = max(0, q - K.dl); j < q; ++j) in = coef_fma(K.pc, in, se[(j << lw) + lc]);
+  float2 *const sb = se + blockDim.x;
+  sb[t] = cn_chunk_backward<Coef, CL>(in, K, y);
+  __syncthreads();
+  in = make_float2(0.0f, 0.0f);
+  for (int j = min(tpl - 1, q + K.dl); j > q; --j) in = coef_fma(K.pc, in, sb[(j << lw) + lc]);
+  cn_chunk_inflow<Coef, CL>(in, K, y);
+  // u_0 of the column is the first chunk's y[0]
+  float2 img = make_float2(0.0f, 0.0f);
+  if (K.dl == 1) {
+    if (q == 0) img = coef_mul(K.al, y[0]);
+  } else {
+    __syncthreads();  // the forward ends have been read
+    if (q == 0) se[lc] = y[0];
+    __syncthreads();
+    if (q < K.dl) {
+      img = coef_mul(K.al, se[lc]);
+      for (int j = 0; j < q; ++j) img = coef_mul(K.pc, img);
+    }
+    __syncthreads();  // before the next tile's forward ends
+  }
+  cn_chunk_finish<Coef, CL>(img, K, y, v);
+}
+
 }  // namespace
 }  // namespace dgpe

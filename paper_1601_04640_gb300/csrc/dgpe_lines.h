@@ -9,6 +9,24 @@
 
 namespace dgpe {
 
+// Launch of a pass that begins with pdl_wait (dgpe_device.cuh).  early: its
+// blocks may start before the kernel ahead of it in the stream has ended.
+template <class... P, class... A>
+inline cudaError_t launch_pdl(bool early, void (*k)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                              const A &...args) {
+  cudaLaunchConfig_t c{};
+  cudaLaunchAttribute a{};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &a;
+  c.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&c, k, static_cast<P>(args)...);
+}
+
 // Constant-coefficient form of one Crank-Nicolson substep along a line
 // (dgpe_lines.cuh): alpha, -2 kt m, alpha^CL and alpha^1 .. alpha^CL, the
 // reach dl of the chunk inflow (1..4 chunks; 0: the coefficients decay too
@@ -32,7 +50,9 @@ struct ColArgs {
   long long es, os;
   unsigned tot, ncols;
   int n, cl;       // points; points per chunk (16, 12 or 10)
+  int nsm;         // SMs, as in cols_grid
   int final_pass, norm;
+  int early;       // launch_pdl
   int dlim;        // chunk reach of the table form (0: all chunks)
   double tau;      // kt = tau (imaginary time) or i tau (real time)
 };
@@ -55,6 +75,7 @@ struct RowArgs {
   const float *vx, *vy, *vz;
   int n, ny, nrows;
   int has_dip;
+  int early;   // launch_pdl
   int src;     // forward: 0 sc^2 |psi|^2, 1 the real field dens_in, 2 sc^2 psi^2 of a real state
   int mode;    // backward: ROWS_*
   double dtf;  // fraction of dt of the exponential substep
@@ -64,6 +85,8 @@ struct RowArgs {
 enum { ROWS_STEP = 0, ROWS_PHI = 1, ROWS_CN = 2, ROWS_EXP = 3, ROWS_REAL = 4, ROWS_MODES = 5 };
 // points of a row that one lane solves: the chunk length of the constant form
 int rows_chunk(int n);
+// rows of a warp's tile
+int rows_per_tile(int n);
 // The grids raise the kernels' shared-memory limits: once before a launch.
 cudaError_t rows_fwd_grid(int n, int nrows, int src, int nsm, int *grid);
 cudaError_t rows_fwd_launch(const RowArgs &A, int grid, cudaStream_t s);

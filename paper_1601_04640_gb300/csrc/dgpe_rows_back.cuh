@@ -24,18 +24,10 @@ template <int CL, bool REAL> struct RowStage {
   }
 };
 
-// The exponential of a lane's CL sites.  The library's sincosf and expm1f are
-// called out of line: inlined at every site they were most of the kernel's
-// code, and a warp that runs it once (a small grid) or out of step with its
-// neighbours waits for instructions.  A lane whose exponents all lie within
+// The exponential of a lane's CL sites.  A lane whose exponents all lie within
 // 1/8 takes the short Taylor series (sin_cosm1, fexpm1), within 2 (1) the
-// series below, whose first omitted terms are below 2e-10 (3e-8) relative.
-__device__ __noinline__ float2 sincosm1_any(float x) {
-  float s, c;
-  sincosf(x * 0.5f, &s, &c);
-  return make_float2(2.0f * s * c, -2.0f * s * s);
-}
-__device__ __noinline__ float expm1_any(float x) { return expm1f(x); }
+// series below, whose first omitted terms are below 2e-10 (3e-8) relative;
+// beyond that the library functions, out of line.
 __device__ __forceinline__ float2 phase_update(float2 v, float sn, float cm1) {  // v e^{-i th}, as in nonlinear_factor
   return make_float2(v.x + (v.x * cm1 + v.y * sn), v.y + (v.y * cm1 - v.x * sn));
 }
@@ -73,8 +65,8 @@ template <int CL> __device__ __forceinline__ void exp_real_time(float2 (&v)[CL],
   } else {
 #pragma unroll
     for (int i = 0; i < CL; ++i) {
-      const float2 e = sincosm1_any(th[i]);
-      v[i] = phase_update(v[i], e.x, e.y);
+      const float2 e = sincos_call(th[i] * 0.5f);
+      v[i] = phase_update(v[i], 2.0f * e.x * e.y, -2.0f * e.x * e.x);
     }
   }
 }
@@ -111,8 +103,55 @@ template <int CL> __device__ __forceinline__ void exp_imag_time(float (&th)[CL])
     }
   } else {
 #pragma unroll
-    for (int i = 0; i < CL; ++i) th[i] = expm1_any(-th[i]);
+    for (int i = 0; i < CL; ++i) th[i] = expm1_call(-th[i]);
   }
+}
+
+// Crank-Nicolson along x: CL consecutive points of a row per lane, TPL lanes
+// per row.
+template <typename Coef, int CL, int TPL>
+__device__ __forceinline__ void row_solve(float2 (&v)[CL], int q, const CnConst<Coef> &K) {
+  float2 y[CL];
+  float2 prev = shfl_up(v[CL - 1], 1, TPL), next = shfl_down(v[0], 1, TPL);
+  if (q == 0) prev = make_float2(0.0f, 0.0f);
+  if (q == TPL - 1) next = make_float2(0.0f, 0.0f);
+  const float2 e = cn_chunk_forward<Coef, CL>(v, prev, next, K, y);
+  float2 in = make_float2(0.0f, 0.0f);
+  for (int d = K.dl; d > 0; --d) {
+    const float2 t = shfl_up(e, d, TPL);
+    if (q >= d) in = coef_fma(K.pc, in, t);
+  }
+  const float2 g = cn_chunk_backward<Coef, CL>(in, K, y);
+  in = make_float2(0.0f, 0.0f);
+  for (int d = K.dl; d > 0; --d) {
+    const float2 t = shfl_down(g, d, TPL);
+    if (q + d < TPL) in = coef_fma(K.pc, in, t);
+  }
+  cn_chunk_inflow<Coef, CL>(in, K, y);
+  // u_0 of the line is the first chunk's y[0]
+  float2 img = make_float2(__shfl_sync(0xffffffffu, y[0].x, 0, TPL), __shfl_sync(0xffffffffu, y[0].y, 0, TPL));
+  img = coef_mul(K.al, img);
+  for (int d = 0; d < K.dl; ++d)
+    if (d < q) img = coef_mul(K.pc, img);
+  if (q >= K.dl) img = make_float2(0.0f, 0.0f);
+  cn_chunk_finish<Coef, CL>(img, K, y, v);
+}
+// C2R of a pair of rows from their staged half spectra: Phi_d of both at the
+// lane's CL consecutive points.  xa, xb: the rows' spectra (in z or elsewhere).
+template <int N> __device__ __forceinline__ void row_c2r(float2 *z, const float2 *xa, const float2 *xb, int q) {
+  constexpr int CL = Row<N>::CL, TPL = Row<N>::TPL;
+  float2 v[CL];
+#pragma unroll
+  for (int r = 0; r < CL; ++r) {
+    // Z = X0 + i X1 of the two rows, extended by X(N - k) = conj X(k)
+    const int a = q + r * TPL;
+    const bool up = r > CL / 2 || (r == CL / 2 && q > 0);  // a > N / 2
+    float2 x = xa[up ? N - a : a], y = xb[up ? N - a : a];
+    if (up) { x.y = -x.y; y.y = -y.y; }
+    if ((r == 0 || r == CL / 2) && q == 0) { x.y = 0.0f; y.y = 0.0f; }  // real ends
+    v[r] = make_float2(x.x - y.y, x.y + y.x);
+  }
+  row_first<N, true>(z, v);
 }
 
 template <int N, int MODE> struct BackCfg {
@@ -187,15 +226,17 @@ __global__ void __launch_bounds__(32 * kRowWarps, Row<N>::BLOCKS)
   // tiles are dealt out block by block, so few tiles spread over the SMs
   int tile = w * gridDim.x + blockIdx.x;
   const int nw = gridDim.x * kRowWarps;
+  row_twiddles<N>(tws, A.tw);
+  if constexpr (EXP)
+    for (int i = threadIdx.x; i < N; i += blockDim.x)
+      reinterpret_cast<float *>(vxs)[((i % CL) / 4 * TPL + i / CL) * 4 + i % 4] = A.vx[i];
+  pdl_wait();
   if (tile < ntiles) {
     if (dip) issue_spec(tile);
     if (B::PSI && lane == 0) issue_psi(tile);
   }
-  row_twiddles<N>(tws, A.tw);
   float dts = 0.0f, gdt = 0.0f, gdddt = 0.0f, sc = 1.0f;
   if constexpr (EXP) {
-    for (int i = threadIdx.x; i < N; i += blockDim.x)
-      reinterpret_cast<float *>(vxs)[((i % CL) / 4 * TPL + i / CL) * 4 + i % 4] = A.vx[i];
     float *const s_k = reinterpret_cast<float *>(smrows + S::off_k);
     if (threadIdx.x == 0) {
       s_k[0] = (float)(trap_dts(A.prm, *A.step) * A.dtf);
@@ -227,20 +268,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, Row<N>::BLOCKS)
         return;
       }
       const float2 *const xa = z + l * C::PS, *const xb = xa + NL * C::PS;
-      {
-        float2 v[CL];
-#pragma unroll
-        for (int r = 0; r < CL; ++r) {
-          // Z = X0 + i X1 of the two rows, extended by X(N - k) = conj X(k)
-          const int a = q + r * TPL;
-          const bool up = r > CL / 2 || (r == CL / 2 && q > 0);  // a > N / 2
-          float2 x = xa[up ? N - a : a], y = xb[up ? N - a : a];
-          if (up) { x.y = -x.y; y.y = -y.y; }
-          if ((r == 0 || r == CL / 2) && q == 0) { x.y = 0.0f; y.y = 0.0f; }  // real ends
-          v[r] = make_float2(x.x - y.y, x.y + y.x);
-        }
-        row_first<N, true>(z, v);
-      }
+      row_c2r<N>(z, xa, xb, q);
       // the state's next tile, once the store of its last one has been read
       if (B::PSI && !first && lane == 0) {
         bulk_wait_read_all();
@@ -280,32 +308,6 @@ __global__ void __launch_bounds__(32 * kRowWarps, Row<N>::BLOCKS)
         }
         return;
       }
-      auto solve = [&](float2(&v)[CL]) {
-        float2 y[CL];
-        float2 prev = shfl_up(v[CL - 1], 1, TPL), next = shfl_down(v[0], 1, TPL);
-        if (q == 0) prev = make_float2(0.0f, 0.0f);
-        if (q == TPL - 1) next = make_float2(0.0f, 0.0f);
-        const float2 e = cn_chunk_forward<Coef, CL>(v, prev, next, K, y);
-        float2 in = make_float2(0.0f, 0.0f);
-        for (int d = K.dl; d > 0; --d) {
-          const float2 t = shfl_up(e, d, TPL);
-          if (q >= d) in = coef_fma(K.pc, in, t);
-        }
-        const float2 g = cn_chunk_backward<Coef, CL>(in, K, y);
-        in = make_float2(0.0f, 0.0f);
-        for (int d = K.dl; d > 0; --d) {
-          const float2 t = shfl_down(g, d, TPL);
-          if (q + d < TPL) in = coef_fma(K.pc, in, t);
-        }
-        cn_chunk_inflow<Coef, CL>(in, K, y);
-        // u_0 of the line is the first chunk's y[0]
-        float2 img = make_float2(__shfl_sync(0xffffffffu, y[0].x, 0, TPL), __shfl_sync(0xffffffffu, y[0].y, 0, TPL));
-        img = coef_mul(K.al, img);
-        for (int d = 0; d < K.dl; ++d)
-          if (d < q) img = coef_mul(K.pc, img);
-        if (q >= K.dl) img = make_float2(0.0f, 0.0f);
-        cn_chunk_finish<Coef, CL>(img, K, y, v);
-      };
       if constexpr (MODE == ROWS_REAL) {
         // the pair's rows are the parts of one complex line: each part scaled
         // by its own row's factor, one solve with the real coefficients
@@ -339,7 +341,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, Row<N>::BLOCKS)
         exp_imag_time<CL>(tb);
 #pragma unroll
         for (int i = 0; i < CL; ++i) v[i] = make_float2(v[i].x + v[i].x * ta[i], v[i].y + v[i].y * tb[i]);
-        solve(v);
+        row_solve<Coef, CL, TPL>(v, q, K);
 #pragma unroll
         for (int c = 0; c < G::NP; ++c) {
           *reinterpret_cast<float4 *>(stage + G::off(ia, c)) =
@@ -382,7 +384,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, Row<N>::BLOCKS)
               for (int i = 0; i < CL; ++i) v[i] = make_float2(v[i].x + v[i].x * th[i], v[i].y + v[i].y * th[i]);
             }
           }
-          if constexpr (CN) solve(v);
+          if constexpr (CN) row_solve<Coef, CL, TPL>(v, q, K);
 #pragma unroll
           for (int c = 0; c < G::NP; ++c)
             *reinterpret_cast<float4 *>(stage + G::off(ic, c)) =
@@ -407,8 +409,7 @@ template <typename Coef, int MODE, class F> cudaError_t with_back(int n, F &&f) 
 template <typename Coef, int MODE>
 cudaError_t back_launch(const RowArgs &A, const CUtensorMap &tm, const CnConst<Coef> &K, int grid, cudaStream_t s) {
   return with_back<Coef, MODE>(A.n, [&](auto k, int smem, int rows) {
-    k<<<grid, 32 * kRowWarps, smem, s>>>(tm, A, K, (A.nrows + rows - 1) / rows);
-    return cudaGetLastError();
+    return launch_pdl(A.early != 0, k, dim3(grid), 32 * kRowWarps, smem, s, tm, A, K, (A.nrows + rows - 1) / rows);
   });
 }
 template <typename Coef, int MODE> cudaError_t back_grid(int n, int nrows, int nsm, int *grid) {

@@ -48,8 +48,9 @@ __global__ void __launch_bounds__(32 * kRowWarps, Row<N>::BLOCKS) k_rows_fwd(con
   // tiles are dealt out block by block, so few tiles spread over the SMs
   int tile = w * gridDim.x + blockIdx.x;
   const int nw = gridDim.x * kRowWarps;
-  if (tile < ntiles) issue(tile);
   row_twiddles<N>(tws, A.tw);
+  pdl_wait();
+  if (tile < ntiles) issue(tile);
   float sc2 = 1.0f;
   if (SRC != 1) {
     const float sc = (float)A.prm[PRM_SC];
@@ -115,11 +116,10 @@ template <class F> cudaError_t with_fwd(int n, int src, F &&f) {
 }  // namespace
 
 int rows_chunk(int n) { return rows_cl(n); }
+int rows_per_tile(int n) { return 64 * rows_cl(n) / n; }
 cudaError_t rows_fwd_launch(const RowArgs &A, int grid, cudaStream_t s) {
   return with_fwd(A.n, A.src, [&](auto k, int smem, int rows) {
-    const int ntiles = (A.nrows + rows - 1) / rows;
-    k<<<grid, 32 * kRowWarps, smem, s>>>(A, ntiles);
-    return cudaGetLastError();
+    return launch_pdl(A.early != 0, k, dim3(grid), 32 * kRowWarps, smem, s, A, (A.nrows + rows - 1) / rows);
   });
 }
 cudaError_t rows_fwd_grid(int n, int nrows, int src, int nsm, int *grid) {
