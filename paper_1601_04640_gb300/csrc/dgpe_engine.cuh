@@ -315,7 +315,6 @@ template <typename R> struct EngineT : Engine {
   // real state (imaginary time): psi holds nx reals per row, viewed by the
   // strided CN passes as nx/2 complex columns (pairs of real lines)
   bool rpsi = false;
-  Cx *ocx = nullptr;  // complex copy of a real state for the observables
 
   ~EngineT() override {
     if (gexec) cudaGraphExecDestroy(gexec);
@@ -325,7 +324,7 @@ template <typename R> struct EngineT : Engine {
                     cntab[0], cntab[1], cntab[2], prm, partial, obs_part, dip_part, obs_out,
                     dstep, counter, stage, adjG, adjT, adj_phi, adj_sig, adj_ksig, adj_part,
                     adj_acc, cntab_adj[0], cntab_adj[1], cntab_adj[2], twf[0], twf[1], twf[2],
-                    twi[0], twi[1], twi[2], ocx};
+                    twi[0], twi[1], twi[2]};
     for (void *b : bufs)
       if (b) cudaFree(b);
     for (Cx *b : ckpts) cudaFree(b);
@@ -498,7 +497,10 @@ template <typename R> struct EngineT : Engine {
       if (fy.T > DGPE_MAXT_FFT || fz.T > DGPE_MAXT_FFT) { err = "strided FFT block too large"; return DGPE_EUNSUPPORTED; }
     }
     // scratch: norm partials, observable partials
-    obs_blocks = (int)std::min<size_t>(152 * 8, (nsites + 255) / 256);
+    // rows per thread of the site sums: as many (to 32) as leave eight warps
+    // per SM scheduler
+    obs_rows = (int)std::max<size_t>(1, std::min<size_t>(32, nsites / 4 / ((size_t)nsm * 4 * 8 * 32)));
+    obs_blocks = (int)(((size_t)(nx / 4) * nz * ((ny + obs_rows - 1) / obs_rows) + 255) / 256);
     const FtCfg &last = (dim == 3) ? fz : fy;
     ndip = has_dip ? (int)(last.grid.x * last.grid.y) : 0;
     const CnCfg &fin = cn[dim == 3 ? 2 : 1];
@@ -510,7 +512,7 @@ template <typename R> struct EngineT : Engine {
                                          cn_serial ? (size_t)lfin.grid.x * lfin.grid.y : (size_t)0})))) return rc;
     if ((rc = dalloc(&obs_part, (size_t)obs_blocks * OBS_COUNT))) return rc;
     if ((rc = dalloc(&dip_part, (size_t)std::max(ndip, 1)))) return rc;
-    if ((rc = dalloc(&obs_out, OBS_COUNT + 1))) return rc;
+    if ((rc = dalloc(&obs_out, OBS_COUNT + 2 + PRM_COUNT))) return rc;
     if ((rc = set_smem_attrs())) return rc;
     setup_lines();
     DGPE_CK(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
@@ -1490,18 +1492,8 @@ template <typename R> struct EngineT : Engine {
   int observables(dgpe_obs *o, cudaStream_t s) override {
     int rc;
     DGPE_LCK("(pending before observables)");
-    // a real state is widened to (psi, 0) first; the sums below then run
-    // unchanged on the complex copy
-    const Cx *obs_psi = psi;
-    if (rpsi) {
-      if (!ocx && (rc = dalloc(&ocx, nsites))) return rc;
-      k_widen_real<R><<<152 * 8, 256, 0, s>>>(ocx, (const R *)psi, nsites);
-      launched(1);
-      DGPE_LCK("widen");
-      obs_psi = ocx;
-    }
     if (has_dip) {
-      if ((rc = launch_forward_spectrum(s, obs_psi))) return rc;
+      if ((rc = launch_forward_spectrum(s))) return rc;
       DGPE_LCK("density/R2C");
       if (dim == 3) {
         if ((rc = launch_fft(fy, 0, s))) return rc;
@@ -1512,22 +1504,20 @@ template <typename R> struct EngineT : Engine {
       DGPE_LCK("spectral energy sum");
     }
     OArgs<R> A{};
-    A.psi = obs_psi; A.prm = prm; A.partial = obs_part; A.nx = nx; A.ny = ny; A.nz = nz; A.dim = dim;
-    A.rows_per_block = 0; A.hx = p.h[0]; A.hy = p.h[1]; A.hz = (dim == 3) ? p.h[2] : 0.0;
+    A.psi = psi; A.prm = prm; A.partial = obs_part; A.nx = nx; A.ny = ny; A.nz = nz; A.dim = dim;
+    A.rows = obs_rows; A.hx = p.h[0]; A.hy = p.h[1]; A.hz = (dim == 3) ? p.h[2] : 0.0;
     A.nux = p.nu[0]; A.nuy = p.nu[1]; A.nuz = (dim == 3) ? p.nu[2] : 0.0;
-    k_obs_sites<R><<<obs_blocks, 256, 0, s>>>(A);
+    if (rpsi) k_obs_sites<R, true><<<obs_blocks, 256, 0, s>>>(A);
+    else k_obs_sites<R, false><<<obs_blocks, 256, 0, s>>>(A);
     launched(1);
     DGPE_LCK("site sums");
-    k_obs_final<<<1, 256, 0, s>>>(obs_part, obs_blocks, dip_part, ndip, obs_out);
+    k_obs_final<<<OBS_COUNT + 1, 256, 0, s>>>(obs_part, obs_blocks, dip_part, ndip, prm, dstep, obs_out);
     launched(1);
     DGPE_LCK("final sums");
-    double h[OBS_COUNT + 1];
-    double hp[PRM_COUNT];
-    long long st = 0;
+    double h[OBS_COUNT + 2 + PRM_COUNT];
     DGPE_CK(cudaMemcpyAsync(h, obs_out, sizeof(h), cudaMemcpyDeviceToHost, s));
-    DGPE_CK(cudaMemcpyAsync(hp, prm, sizeof(hp), cudaMemcpyDeviceToHost, s));
-    DGPE_CK(cudaMemcpyAsync(&st, dstep, sizeof(st), cudaMemcpyDeviceToHost, s));
     DGPE_CK(cudaStreamSynchronize(s));
+    const double *const hp = h + OBS_COUNT + 1;
     if (hp[PRM_TIMEOUT] != 0.0) {
       err = "a bounded device-side wait ran out (the step's results are incomplete)";
       return DGPE_ETIMEOUT;
@@ -1537,7 +1527,7 @@ template <typename R> struct EngineT : Engine {
       return DGPE_ENONFINITE;
     }
     const double cell = hp[PRM_CELL];
-    const double t = (double)st * p.dt;
+    const double t = hp[PRM_COUNT] * p.dt;
     double sm = 1.0;
     for (int m = 1; m <= (int)hp[PRM_M]; ++m) sm += hp[PRM_CM + m - 1] * std::sin((double)m * t);
     const double norm = cell * h[OBS_N];
