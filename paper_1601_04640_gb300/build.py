@@ -17,7 +17,7 @@ LIB = os.path.join(HERE, "libdgpe.so")
 PLAIN_LIB = os.path.join(HERE, "libdgpe_plain.so")
 PLAIN_SRC = os.path.join(CSRC, "plain", "dgpe_plain.cu")
 UNITS = ["dgpe_api.cu", "dgpe_f64.cu", "dgpe_f32.cu", "dgpe_noalloc.cu", "dgpe_batch.cu", "dgpe_cols.cu",
-         "dgpe_rows_fwd.cu", "dgpe_rows_real.cu", "dgpe_rows_cplx.cu"]
+         "dgpe_rows_fwd.cu", "dgpe_rows_real.cu", "dgpe_rows_cplx.cu", "dgpe_fine.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-I", CSRC, "-I", os.path.join(ROOT, "include")]

@@ -612,8 +612,9 @@ __device__ __forceinline__ void pdl_wait() {
 // accesses on distinct banks).
 template <typename R, typename Coef, int CL>
 __device__ __forceinline__ void cn_line(cx<R> *line, int n, int TPL, int q, Coef kt,
-                                        const Coef *__restrict__ tab, bool active) {
+                                        const Coef *__restrict__ tab, bool active, int dlim = 0) {
   typedef cx<R> Cx;
+  const int DL = (dlim > 0 && dlim < TPL) ? dlim : TPL;  // scan rounds, as in cn_line_st
   const Coef *tm = tab, *ta = tab + n, *tp = tab + 2 * n, *tq = tab + 3 * n;
   const int a0 = q * CL;
   Cx y[CL];
@@ -637,7 +638,7 @@ __device__ __forceinline__ void cn_line(cx<R> *line, int n, int TPL, int q, Coef
   // inclusive scan over the chunks (lane segment of width TPL)
   Coef P = active ? tp[a0 + CL - 1] : coef_zero<Coef>();
   Cx Y = acc;
-  for (int d = 1; d < TPL; d <<= 1) {
+  for (int d = 1; d < DL; d <<= 1) {
     Coef Pn = shfl_up(P, d, TPL);
     Cx Yn = shfl_up(Y, d, TPL);
     if (q >= d) { Y = Y + coef_mul(P, Yn); P = coef_prod(P, Pn); }
@@ -659,7 +660,7 @@ __device__ __forceinline__ void cn_line(cx<R> *line, int n, int TPL, int q, Coef
   }
   Coef Q = active ? tq[a0] : coef_zero<Coef>();
   Cx W = acc;
-  for (int d = 1; d < TPL; d <<= 1) {
+  for (int d = 1; d < DL; d <<= 1) {
     Coef Qn = shfl_down(Q, d, TPL);
     Cx Wn = shfl_down(W, d, TPL);
     if (q + d < TPL) { W = W + coef_mul(Q, Wn); Q = coef_prod(Q, Qn); }

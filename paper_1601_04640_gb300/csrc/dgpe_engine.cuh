@@ -15,6 +15,7 @@
 #include "dgpe.h"
 #include "dgpe_kernels.cuh"
 #include "dgpe_lines.h"
+#include "dgpe_fine.h"
 
 namespace dgpe {
 
@@ -203,6 +204,18 @@ constexpr size_t kEarlySites = (size_t)1 << 18;
 // largest grid with a graph of several steps: above it a step takes some 100 us,
 // beside which the gap between two graphs is small
 constexpr size_t kRunSites = (size_t)1 << 22;
+// Largest FP64 grid that takes the passes of dgpe_fine.cu (us per step in real
+// time, the other passes first): 64 x 64 x 48 191 -> 109, 64 x 80 x 64 250 ->
+// 172, 96^3 465 -> 420, but 128 x 96 x 96 512 -> 540: up to 2^20 sites.  Where
+// every length is a power of two up to 128 the other passes' FMA-form
+// transforms win from 2^18 (64^3 184 -> 196, 128 x 128 x 64 463 -> 472); where
+// nx is 5 2^k their 20 points per thread spill and they lose to the end of the
+// range (160^3 2239 -> 1950).
+inline size_t fine_sites(int nx, int ny, int nz) {
+  auto small2 = [](int n) { return is_pow2(n) && n <= 128; };
+  if (nx % 5 == 0) return (size_t)1 << 23;
+  return small2(nx) && small2(ny) && small2(nz) && nz > 1 ? ((size_t)1 << 18) - 1 : (size_t)1 << 20;
+}
 // Call f(N, EPT) for any line length of the FP32 strided transforms (EPT
 // elements per thread: 16, 12 or 20 for 2^k, 3 2^k, 5 2^k).
 template <class F> int with_col_len(int n, F &&f) {
@@ -221,6 +234,12 @@ template <typename R> struct EngineT : Engine {
   typedef cx<R> Cx;
   static constexpr int EPT_S = sizeof(R) == 8 ? DGPE_EPT_S_F64 : 16;  // strided FFTs, power-of-two lengths
   int var[3] = {VAR_P2, VAR_P2, VAR_P2};           // kernel variant per axis
+  // FP64 on a small grid: the passes of dgpe_fine.cu, with the constant CN form
+  // of each axis (imaginary, real time, conjugated) and its correction tables
+  bool fine = false;
+  FineCn<double> fine_kr[3] = {};
+  FineCn<double2> fine_kc[3] = {}, fine_ka[3] = {};
+  double2 *fineE = nullptr;
   static constexpr int PW = 128 / (int)sizeof(Cx); // pad period of line-major tiles
   static constexpr int W = 128 / (int)sizeof(Cx);  // columns per strided tile (128 B)
 
@@ -323,7 +342,7 @@ template <typename R> struct EngineT : Engine {
     void *bufs[] = {psi, spec, U, phi_tmp, tw[0], tw[1], tw[2], vt[0], vt[1], vt[2],
                     cntab[0], cntab[1], cntab[2], prm, partial, obs_part, dip_part, obs_out,
                     dstep, counter, stage, adjG, adjT, adj_phi, adj_sig, adj_ksig, adj_part,
-                    adj_acc, cntab_adj[0], cntab_adj[1], cntab_adj[2], twf[0], twf[1], twf[2],
+                    adj_acc, cntab_adj[0], cntab_adj[1], cntab_adj[2], fineE, twf[0], twf[1], twf[2],
                     twi[0], twi[1], twi[2]};
     for (void *b : bufs)
       if (b) cudaFree(b);
@@ -377,6 +396,7 @@ template <typename R> struct EngineT : Engine {
       DGPE_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     }
     early = nsites <= kEarlySites;
+    fine = sizeof(R) == 8 && !(p.flags & DGPE_FLAG_CN_SERIAL) && nsites <= fine_sites(nx, ny, nz);
     for (int a = 0; a < dim; ++a) {
       var[a] = axis_variant(nsz[a]);
       if (var[a] == VAR_NONE) {
@@ -509,7 +529,9 @@ template <typename R> struct EngineT : Engine {
     // the pass with half-width tiles; the FP32 pass narrows its tiles to at
     // most 2 nsm of them)
     if ((rc = dalloc(&partial, std::max({2 * (size_t)fin.grid.x * fin.grid.y, 2 * (size_t)nsm + 2,
-                                         cn_serial ? (size_t)lfin.grid.x * lfin.grid.y : (size_t)0})))) return rc;
+                                         cn_serial ? (size_t)lfin.grid.x * lfin.grid.y : (size_t)0,
+                                         fine ? (size_t)fine_cn_blocks(fin.n, fin.ncols * (int)fin.grid.y, nsm) : (size_t)0}))))
+      return rc;
     if ((rc = dalloc(&obs_part, (size_t)obs_blocks * OBS_COUNT))) return rc;
     if ((rc = dalloc(&dip_part, (size_t)std::max(ndip, 1)))) return rc;
     if ((rc = dalloc(&obs_out, OBS_COUNT + 2 + PRM_COUNT))) return rc;
@@ -540,7 +562,7 @@ template <typename R> struct EngineT : Engine {
       cn_serial = false;
     } else if (p.flags & DGPE_FLAG_CN_SERIAL) cn_serial = true;
     else if (p.flags & DGPE_FLAG_CN_CHUNKED) cn_serial = false;
-    else cn_serial = lines_min >= 8192;
+    else cn_serial = lines_min >= 8192 && !fine;
     const int ns[3] = {nx, ny, nz};
     for (int a = 0; a < dim; ++a) {
       LnCfg &L = ln[a];
@@ -635,6 +657,110 @@ template <typename R> struct EngineT : Engine {
     return K;
   }
 
+  // FP64 on a small grid: constants of axis a for kt, and for its conjugate in
+  // real time.  dl chunks reach to below 2^-62 of the largest chunk value.
+  template <typename Coef> void fine_const(int n, zd kt, FineCn<Coef> &K, std::vector<double2> &tab, size_t at) {
+    const int cl = fine_chunk(n), tpl = n / cl;
+    const zd m = 2.0 / (1.0 + 2.0 * kt + std::sqrt(1.0 + 4.0 * kt)), al = kt * m;
+    auto put = [](Coef &c, zd v) {
+      if constexpr (std::is_same<Coef, double2>::value) { c.x = v.real(); c.y = v.imag(); }
+      else c = v.real();
+    };
+    K = FineCn<Coef>{};
+    put(K.al, al);
+    put(K.m2, -2.0 * kt * m);
+    zd p = 1.0;
+    for (int i = 0; i < cl; ++i) { p *= al; put(K.pw[i], p); }
+    const double rho = std::abs(p);
+    for (int k = 0; k < FINE_LOG; ++k) { put(K.pc[k], p); p *= p; }
+    for (int d = 1; d <= std::min<int>(FINE_DL, tpl); ++d)
+      if (std::pow(rho, d) <= 0x1p-62 * (1.0 - rho)) { K.dl = d; break; }
+    const zd den = 1.0 - std::pow(al, 2 * n + 2);
+    Coef *const e = reinterpret_cast<Coef *>(tab.data() + at);
+    for (int i = 0; i < n; ++i) {
+      const zd v = (std::pow(al, i + 2) - std::pow(al, 2 * n - i + 2)) / den;
+      put(e[i], v);
+      if (std::abs(v) > 0x1p-62) K.nE = i / cl + 1;
+    }
+    K.E = reinterpret_cast<const Coef *>(fineE + at);
+  }
+  int build_fine() {
+    const int ns[3] = {nx, ny, nz};
+    const size_t tot = 2 * (size_t)(nx + ny + nz);
+    std::vector<double2> tab(tot);
+    if (!fineE) {
+      int rc = dalloc(&fineE, tot);
+      if (rc) return rc;
+    }
+    size_t at = 0;
+    for (int a = 0; a < dim; ++a, at += 2 * (size_t)ns[a - 1]) {
+      if (imag) {
+        fine_const(ns[a], zd(tau[a], 0.0), fine_kr[a], tab, at);
+      } else {
+        fine_const(ns[a], zd(0.0, tau[a]), fine_kc[a], tab, at);
+        fine_const(ns[a], zd(0.0, -tau[a]), fine_ka[a], tab, at + ns[a]);
+      }
+    }
+    return upload(fineE, tab);
+  }
+  // FP64 on a small grid; false: another kernel runs this pass
+  FineArgs fargs() const {
+    FineArgs A{};
+    if constexpr (sizeof(R) == 8) {
+      A.psi = psi; A.spec = spec; A.phi_out = phi_tmp; A.U = U; A.prm = prm; A.partial = partial; A.step = dstep;
+      A.counter = counter; A.tw = tw[0]; A.vx = vt[0]; A.vy = vt[1]; A.vz = vt[2];
+      A.nx = nx; A.ny = ny; A.nrows = nrows; A.px = px; A.has_dip = has_dip ? 1 : 0; A.nsm = nsm; A.early = early ? 1 : 0;
+    }
+    return A;
+  }
+  bool fine_forward(cudaStream_t s, const Cx *src, const R *dens_in, cudaError_t &e) {
+    if constexpr (sizeof(R) == 8) {
+      if (!fine) return false;
+      FineArgs A = fargs();
+      if (src) A.psi = const_cast<Cx *>(src);
+      A.dens_in = dens_in;
+      e = fine_dens(A, dens_in ? 1 : (rpsi && !src) ? 2 : 0, s);
+      return true;
+    }
+    return false;
+  }
+  bool fine_strided(const FtCfg &f, int mode, cudaStream_t s, cudaError_t &e) {
+    if constexpr (sizeof(R) == 8) {
+      if (!fine || mode > 2) return false;
+      FineArgs A = fargs();
+      A.tw = tw[f.axis]; A.n = f.n; A.ncols = ncol_spec; A.outer = (int)f.grid.y; A.es = f.es; A.os = f.os;
+      e = fine_fft(A, mode, s);
+      return true;
+    }
+    return false;
+  }
+  bool fine_p1(int mode, cudaStream_t s, R *phi_out, cudaError_t &e) {
+    if constexpr (sizeof(R) == 8) {
+      if (!fine || mode > 1) return false;
+      FineArgs A = fargs();
+      if (phi_out) A.phi_out = phi_out;
+      if (mode == 1) e = fine_phi(A, s);
+      else if (imag) e = fine_back(A, fine_kr[0], rpsi, s);
+      else e = fine_back(A, fine_kc[0], s);
+      return true;
+    }
+    return false;
+  }
+  bool fine_solve(int axis, bool final_pass, cudaStream_t s, Cx *buf, bool adjoint, cudaError_t &e) {
+    if constexpr (sizeof(R) == 8) {
+      if (!fine) return false;
+      const CnCfg &c = cn[axis];
+      FineArgs A = fargs();
+      if (buf) A.psi = buf;
+      A.n = c.n; A.ncols = c.ncols; A.outer = (int)c.grid.y; A.es = c.es; A.os = c.os;
+      A.final_pass = final_pass ? 1 : 0; A.norm = (final_pass && imag) ? 1 : 0;
+      if (imag) e = fine_cn(A, fine_kr[axis], s);
+      else e = fine_cn(A, adjoint ? fine_ka[axis] : fine_kc[axis], s);
+      return true;
+    }
+    return false;
+  }
+
   // Crank-Nicolson LU and chunk-scan tables for axis a: m, alpha, P, Q (n
   // each), then the middle-row pivot mu of the two-ended elimination.
   int build_cn_tables() {
@@ -665,12 +791,14 @@ template <typename R> struct EngineT : Engine {
       }
       // scan rounds d < dl reach dl chunks back; what they drop is at most
       // rho^dl / (1 - rho) of the largest chunk value: keep it below 2^-32
+      // (FP64: 2^-62)
+      const double lim = sizeof(R) == 8 ? 0x1p-62 : 0x1p-32;
       int dl = 1;
       if (rho >= 0.5) {
         dl = 0;  // all rounds
       } else {
         double e = rho;
-        while (dl < 64 && e / (1.0 - rho) > 0x1p-32) { e *= e; dl <<= 1; }
+        while (dl < 64 && e / (1.0 - rho) > lim) { e *= e; dl <<= 1; }
         if (dl >= 64) dl = 0;
       }
       cn_dlim[a] = dl;
@@ -719,6 +847,7 @@ template <typename R> struct EngineT : Engine {
         DGPE_CK(cudaMemcpy(cntab[a], t.data(), sizeof(Cx) * t.size(), cudaMemcpyHostToDevice));
       }
     }
+    if (fine) return build_fine();
     return DGPE_OK;
   }
 
@@ -1000,6 +1129,12 @@ template <typename R> struct EngineT : Engine {
     }
   }
   int launch_fft(const FtCfg &f, int mode, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    if (fine_strided(f, mode, s, e)) {
+      launched(1);
+      DGPE_CK(e);
+      return DGPE_OK;
+    }
     SArgs<R> A = sargs(f);
     if (launch_fft_tma(f, mode, A, s) || launch_fft_ct(f, mode, A, s)) {
       launched(1);
@@ -1098,6 +1233,12 @@ template <typename R> struct EngineT : Engine {
   int launch_cn(int axis, bool final_pass, cudaStream_t s, Cx *buf = nullptr, bool adjoint = false) {
     if (cn_serial) return launch_lines(axis, final_pass, s, buf, adjoint);
     if constexpr (sizeof(R) == 4) return launch_cols(axis, final_pass, s, buf, adjoint);
+    cudaError_t e = cudaSuccess;
+    if (fine_solve(axis, final_pass, s, buf, adjoint, e)) {
+      launched(1);
+      DGPE_CK(e);
+      return DGPE_OK;
+    }
     const CnCfg &c = cn[axis];
     CArgs<R> A{};
     A.psi = buf ? buf : psi; A.cntab = adjoint ? cntab_adj[axis] : cntab[axis];
@@ -1137,7 +1278,7 @@ template <typename R> struct EngineT : Engine {
   // density (of `src`, or the real field `dens_in`) -> half spectrum along x
   int launch_forward_spectrum(cudaStream_t s, const Cx *src = nullptr, const R *dens_in = nullptr) {
     cudaError_t e = cudaSuccess;
-    if (launch_rows_fwd(s, src, dens_in, e)) {
+    if (fine_forward(s, src, dens_in, e) || launch_rows_fwd(s, src, dens_in, e)) {
       launched(1);
       DGPE_CK(e);
       return DGPE_OK;
@@ -1165,7 +1306,7 @@ template <typename R> struct EngineT : Engine {
   int launch_p1(int mode, cudaStream_t s, Cx *buf = nullptr, R *phi_out = nullptr, double dtf = 1.0) {
     if (mode == 2 && cn_serial) return launch_lines(0, false, s, buf, true);
     cudaError_t e = cudaSuccess;
-    if (launch_rows_back(mode, s, buf, phi_out, dtf, e)) {
+    if (fine_p1(mode, s, phi_out, e) || launch_rows_back(mode, s, buf, phi_out, dtf, e)) {
       launched(1);
       DGPE_CK(e);
       return DGPE_OK;

@@ -512,7 +512,7 @@ __device__ __forceinline__ void c2r_x_exp_cnx_body(const XArgs<R> &A, int bx) {
   const int l = t / TPLr, q = t - l * TPLr;
   const bool active = RS ? (l < LP && 2 * (p0 + l) < nrows) : (2 * p0 + l) < nrows;
   if constexpr (TAB) cn_line<R, Coef, CL>(pt + l * P, n, TPLr, q, make_kt<Coef>(A.tau),
-                                      reinterpret_cast<const Coef *>(A.cntab), active);
+                                      reinterpret_cast<const Coef *>(A.cntab), active, A.cnd);
   else cn_line_st<R, Coef, CL>(pt + l * P, n, TPLr, q, make_kt<Coef>(A.tau), s_tab, active, A.cnd);
   __syncthreads();
   if constexpr (RS) {
@@ -990,7 +990,7 @@ __device__ __forceinline__ void cn_strided_body(const CArgs<R> &A, int bx, int b
   }
   const int l = threadIdx.x / TPL, q = threadIdx.x - l * TPL;
   if constexpr (TAB) cn_line<R, Coef, CL>(tile + l * P, n, TPL, q, make_kt<Coef>(A.tau),
-                                      reinterpret_cast<const Coef *>(A.cntab), c0 + l < A.ncols);
+                                      reinterpret_cast<const Coef *>(A.cntab), c0 + l < A.ncols, A.cnd);
   else cn_line_st<R, Coef, CL>(tile + l * P, n, TPL, q, make_kt<Coef>(A.tau), s_tab, c0 + l < A.ncols, A.cnd);
   __syncthreads();
   double acc = 0.0;

@@ -13,12 +13,16 @@
 // The array below stays resident on every GPU that loads this library until
 // the process exits.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <mutex>
+#include <type_traits>
 
 #include "dgpe.h"
 #include "dgpe_kernels.cuh"
+#include "dgpe_fine.h"
+#include "dgpe_lines.h"
 
 namespace dgpe {
 namespace {
@@ -45,7 +49,7 @@ size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 // [z][y][kx] (pitch px), and the parameter block (sc = 1, everything else 0).
 // FP64 work at 64 cycles per warp instruction and scheduler is what this costs:
 // U depends on |ky| and |kz| alone, so each value is computed once and written
-// to its two (2D) or four (3D) places, from wavenumber steps dq = 2 pi / (n h)
+// to its two (2D) or four (3D) places (64^3: the whole call 104 -> 60 us), from wavenumber steps dq = 2 pi / (n h)
 // and the factor 1 / N that the host forms; one division (3D) is left.
 template <typename R>
 __global__ void k_noalloc_tables(cx<R> *tw0, cx<R> *tw1, cx<R> *tw2, R *U, double *prm,
@@ -93,97 +97,155 @@ __global__ void k_noalloc_tables(cx<R> *tw0, cx<R> *tw1, cx<R> *tw2, R *U, doubl
 
 bool pow2_in_range(int n) { return n >= 32 && n <= 512 && (n & (n - 1)) == 0; }
 
-bool make_plan_pow2(int n, int ept, FftPlan &pl) {
-  pl.n = n;
-  pl.ns = 0;
-  int m = n;
-  for (int R : {16, 8, 4, 2})
-    while (m % R == 0 && ept % R == 0) { pl.rad[pl.ns++] = R; m /= R; }
-  return m == 1;
+// The chain behind the table kernel: density + R2C along x, the transforms
+// along y and z, C2R along x.
+struct Chain {
+  int dim, nx, ny, nz, nrows, px, ncols, nsm;
+  const void *psi;
+  void *phi, *spec, *U, *tw[3];
+  double *prm;
+  long long *step;
+};
+
+// FP32: the solver's warp-per-tile row passes and length-specialised strided
+// transforms (64^3: 60 -> 27 us against runtime lengths, one launch after the
+// other).  The row kernels' grids (blocks that fit times SMs, and the
+// shared-memory limit that goes with them) depend on the device and the
+// length alone and are found once per device.
+template <int MODE> cudaError_t strided32(const Chain &c, int n, long long es, long long os, int outer, const void *tw,
+                                          cudaStream_t s) {
+  constexpr int E = 16;
+  SArgs<float> A{};
+  A.spec = (float2 *)c.spec; A.U = (float *)c.U; A.tw = (const float2 *)tw; A.estride = es; A.ostride = os;
+  A.n = n; A.ncols = c.ncols; A.nxh = c.nx / 2;
+  auto go = [&](auto Nc) {
+    constexpr int N = decltype(Nc)::value, W = N == 512 ? 8 : 16;
+    return launch_pdl(true, k_fft_strided_ct<E, MODE, N, W>, dim3((c.ncols + W - 1) / W, outer), W * N / E,
+                      sizeof(float2) * N * W, s, A);
+  };
+  switch (n) {
+    case 32: return go(std::integral_constant<int, 32>{});
+    case 64: return go(std::integral_constant<int, 64>{});
+    case 128: return go(std::integral_constant<int, 128>{});
+    case 256: return go(std::integral_constant<int, 256>{});
+    default: return go(std::integral_constant<int, 512>{});
+  }
+}
+// The density pass of a state that bulk copies cannot start at.
+cudaError_t dens_any(const Chain &c, cudaStream_t s) {
+  constexpr int EPT = 8, CL = 16, PW = 128 / (int)sizeof(float2);
+  XArgs<float> X{};
+  X.psi = (float2 *)c.psi; X.spec = (float2 *)c.spec; X.prm = c.prm; X.tw = (const float2 *)c.tw[0];
+  X.nx = c.nx; X.ny = c.ny; X.nrows = c.nrows; X.px = c.px; X.TPL = c.nx / CL; X.C = CL;
+  X.LP = DGPE_MAXT / 2 / X.TPL;
+  X.pitchz = c.nx + c.nx / PW + 1;
+  X.pl.n = c.nx;
+  for (int m = c.nx; m > 1; m /= X.pl.rad[X.pl.ns++]) X.pl.rad[X.pl.ns] = m % 8 == 0 ? 8 : m % 4 == 0 ? 4 : 2;
+  const int npairs = (c.nrows + 1) / 2;
+  const size_t sm = sizeof(float2) * (size_t)X.LP * X.pitchz;  // at most 18 KB
+  k_dens_r2c_x<float, EPT><<<(npairs + X.LP - 1) / X.LP, 2 * X.LP * X.TPL, sm, s>>>(X);
+  return cudaGetLastError();
+}
+cudaError_t chain32(const Chain &c, int dev, cudaStream_t s) {
+  static std::atomic<int> fwd[kMaxDevices][5], back[kMaxDevices][5];  // largest grids, 0: not yet known
+  int k = 0;
+  while ((32 << k) < c.nx) ++k;
+  cudaError_t e;
+  const int all = 1 << 30;
+  int gf = fwd[dev][k].load(), gb = back[dev][k].load();
+  if (!gf) {
+    if ((e = rows_fwd_grid(c.nx, all, 0, c.nsm, &gf)) != cudaSuccess) return e;
+    fwd[dev][k].store(gf);
+  }
+  if (!gb) {
+    if ((e = rows_back_grid_real(c.nx, all, ROWS_PHI, c.nsm, &gb)) != cudaSuccess) return e;
+    back[dev][k].store(gb);
+  }
+  RowArgs A{};
+  A.psi = (float2 *)c.psi; A.spec = (float2 *)c.spec; A.phi_out = (float *)c.phi; A.prm = c.prm; A.step = c.step;
+  A.tw = (const float2 *)c.tw[0]; A.n = c.nx; A.ny = c.ny; A.nrows = c.nrows; A.has_dip = 1;
+  const int tiles = (c.nrows + rows_per_tile(c.nx) - 1) / rows_per_tile(c.nx);
+  if (((uintptr_t)c.psi & 15) == 0) {
+    if ((e = rows_fwd_launch(A, std::min(gf, tiles), s)) != cudaSuccess) return e;
+  } else if ((e = dens_any(c, s)) != cudaSuccess) {
+    return e;
+  }
+  const long long py = c.px, pz = (long long)c.ny * c.px;
+  if (c.dim == 3) {
+    if ((e = strided32<0>(c, c.ny, py, pz, c.nz, c.tw[1], s)) != cudaSuccess) return e;
+    if ((e = strided32<2>(c, c.nz, pz, py, c.ny, c.tw[2], s)) != cudaSuccess) return e;
+    if ((e = strided32<1>(c, c.ny, py, pz, c.nz, c.tw[1], s)) != cudaSuccess) return e;
+  } else if ((e = strided32<2>(c, c.ny, py, pz, 1, c.tw[1], s)) != cudaSuccess) {
+    return e;
+  }
+  A.mode = ROWS_PHI;
+  A.early = 1;
+  return rows_back_launch(A, CUtensorMap{}, CnConst<float>{}, std::min(gb, tiles), s);
 }
 
-template <typename K> cudaError_t smem_attr(K kernel, size_t bytes) {
-  cudaError_t e = cudaSuccess;
-  if (bytes > 48 * 1024) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  return e;
+// FP64: the solver's passes for small grids.
+cudaError_t chain64(const Chain &c, cudaStream_t s) {
+  FineArgs A{};
+  A.psi = (double2 *)c.psi; A.spec = (double2 *)c.spec; A.phi_out = (double *)c.phi; A.U = (double *)c.U;
+  A.prm = c.prm; A.step = c.step; A.tw = (const double2 *)c.tw[0];
+  A.nx = c.nx; A.ny = c.ny; A.nrows = c.nrows; A.px = c.px; A.ncols = c.ncols; A.has_dip = 1; A.nsm = c.nsm;
+  cudaError_t e = fine_dens(A, 0, s);  // reads what the table kernel wrote: not early
+  A.early = 1;
+  auto strided = [&](int mode, int axis) {
+    if (e != cudaSuccess) return;
+    FineArgs B = A;
+    const long long py = c.px, pz = (long long)c.ny * c.px;
+    B.tw = (const double2 *)c.tw[axis];
+    B.n = axis == 1 ? c.ny : c.nz; B.es = axis == 1 ? py : pz; B.os = axis == 1 ? pz : py; B.outer = axis == 1 ? c.nz : c.ny;
+    e = fine_fft(B, mode, s);
+  };
+  if (c.dim == 3) {
+    strided(0, 1);
+    strided(2, 2);
+    strided(1, 1);
+  } else {
+    strided(2, 1);
+  }
+  return e == cudaSuccess ? fine_phi(A, s) : e;
 }
 
 template <typename R>
 int run(const void *psi, void *phi, int dim, const int *n, const double *h, int kernel, double qd,
-        cudaStream_t s, unsigned char *base) {
+        cudaStream_t s, int dev, unsigned char *base) {
   typedef cx<R> Cx;
-  constexpr int EPT_X = 8, EPT_S = sizeof(R) == 8 ? 8 : 16, CL = 16;
-  constexpr int W = 128 / (int)sizeof(Cx), PW = 128 / (int)sizeof(Cx);
-  const int nx = n[0], ny = n[1], nz = (dim == 3) ? n[2] : 1;
-  const int nrows = ny * nz;
-  int px = nx / 2 + 1;
-  if (sizeof(Cx) == 8) px = (px + 1) & ~1;
-  const int ncols = nx / 2 + 1;
-  const size_t nspec = (size_t)px * nrows;
+  Chain c{};
+  c.dim = dim; c.psi = psi; c.phi = phi;
+  c.nx = n[0]; c.ny = n[1]; c.nz = (dim == 3) ? n[2] : 1;
+  c.nrows = c.ny * c.nz;
+  c.px = c.nx / 2 + 1;
+  if (sizeof(Cx) == 8) c.px = (c.px + 1) & ~1;
+  c.ncols = c.nx / 2 + 1;
   // carve the scratch array
   size_t off = 0;
-  Cx *spec = (Cx *)(base + off); off = align256(off + nspec * sizeof(Cx));
-  R *U = (R *)(base + off); off = align256(off + nspec * sizeof(R));
-  Cx *tw[3];
-  for (int a = 0; a < 3; ++a) { tw[a] = (Cx *)(base + off); off = align256(off + 512 * sizeof(Cx)); }
-  double *prm = (double *)(base + off); off = align256(off + PRM_COUNT * sizeof(double));
-  long long *step = (long long *)(base + off); off = align256(off + sizeof(long long));
+  auto carve = [&](size_t bytes) { void *p = base + off; off = align256(off + bytes); return p; };
+  const size_t nspec = (size_t)c.px * c.nrows;
+  c.spec = carve(nspec * sizeof(Cx));
+  c.U = carve(nspec * sizeof(R));
+  for (int a = 0; a < 3; ++a) c.tw[a] = carve(512 * sizeof(Cx));
+  c.prm = (double *)carve(PRM_COUNT * sizeof(double));
+  c.step = (long long *)carve(sizeof(long long));
   if (off > kScratchBytes) { set_err("grid too large for the static scratch array"); return DGPE_EUNSUPPORTED; }
-
-  FftPlan plx, ply, plz;
-  if (!make_plan_pow2(nx, EPT_X, plx) || !make_plan_pow2(ny, EPT_S, ply) ||
-      (dim == 3 && !make_plan_pow2(nz, EPT_S, plz))) {
-    set_err("unsupported grid size");
-    return DGPE_EUNSUPPORTED;
-  }
-  // x-line configuration (same rules as the solver's)
-  const int TPL = nx / CL;
-  const int LP = std::max(1, (sizeof(R) == 8 ? 64 : DGPE_MAXT / 2) / TPL);
-  const int T = 2 * LP * TPL;
-  const int pitchz = nx + nx / PW + 1, pitch = nx + nx / CL + 1;
-  const size_t xsm = sizeof(Cx) * (size_t)(LP * pitchz + 2 * LP * pitch);
-  const int xgrid = ((nrows + 1) / 2 + LP - 1) / LP;
-
-  cudaError_t e;
-  if ((e = smem_attr(k_dens_r2c_x<R, EPT_X>, xsm)) != cudaSuccess ||
-      (e = smem_attr(k_c2r_x_exp_cnx<R, R, EPT_X, CL, 1>, xsm)) != cudaSuccess) {
-    set_err("cudaFuncSetAttribute", cudaGetErrorString(e));
-    return DGPE_ECUDA;
-  }
-  {
+  cudaError_t e = cudaDeviceGetAttribute(&c.nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) {
     const double twopi = 6.283185307179586476925286766559, hz = dim == 3 ? h[2] : 1.0;
     const double pref = kernel == DGPE_KERNEL_DIPOLAR_3D ? 4.0 * M_PI / 3.0 : (4.0 * M_PI / 3.0) / (sqrt(2.0 * M_PI) * qd);
-    const int cnt = (nx / 2 + 1) * (ny / 2 + 1) * (nz / 2 + 1);
-    k_noalloc_tables<R><<<std::min((cnt + 63) / 64, 152 * 8), 64, 0, s>>>(
-        tw[0], tw[1], tw[2], U, prm, step, dim, nx, ny, nz, px, twopi / (nx * h[0]), twopi / (ny * h[1]), twopi / (nz * hz),
-        kernel, qd, pref, 1.0 / ((double)nx * ny * nz));
+    const int cnt = (c.nx / 2 + 1) * (c.ny / 2 + 1) * (c.nz / 2 + 1);
+    k_noalloc_tables<R><<<std::min((cnt + 63) / 64, c.nsm * 8), 64, 0, s>>>(
+        (Cx *)c.tw[0], (Cx *)c.tw[1], (Cx *)c.tw[2], (R *)c.U, c.prm, c.step, dim, c.nx, c.ny, c.nz, c.px,
+        twopi / (c.nx * h[0]), twopi / (c.ny * h[1]), twopi / (c.nz * hz), kernel, qd, pref,
+        1.0 / ((double)c.nx * c.ny * c.nz));
+    e = cudaGetLastError();
   }
-  XArgs<R> X{};
-  X.psi = (Cx *)psi; X.spec = spec; X.phi_out = (R *)phi; X.prm = prm; X.step = step;
-  X.tw = tw[0]; X.pl = plx; X.nx = nx; X.ny = ny; X.nrows = nrows; X.px = px; X.LP = LP;
-  X.pitchz = pitchz; X.pitch = pitch; X.TPL = TPL; X.C = CL; X.has_dip = 1;
-  k_dens_r2c_x<R, EPT_X><<<xgrid, T, xsm, s>>>(X);
-  auto strided = [&](int mode, int nn, long long es, long long os, int outer, const FftPlan &pl, const Cx *t) {
-    const int w = std::max(1, std::min(W, DGPE_MAXT * EPT_S / nn));
-    SArgs<R> A{};
-    A.spec = spec; A.U = U; A.tw = t; A.pl = pl; A.estride = es; A.ostride = os; A.n = nn;
-    A.ncols = ncols; A.W = w; A.nxh = nx / 2;
-    dim3 grid((ncols + w - 1) / w, outer);
-    const int TT = w * nn / EPT_S;
-    const size_t sm = sizeof(Cx) * (size_t)nn * w;
-    if (mode == 0) k_fft_strided<R, EPT_S, 0><<<grid, TT, sm, s>>>(A);
-    else if (mode == 1) k_fft_strided<R, EPT_S, 1><<<grid, TT, sm, s>>>(A);
-    else k_fft_strided<R, EPT_S, 2><<<grid, TT, sm, s>>>(A);
-  };
-  if (dim == 3) {
-    strided(0, ny, px, (long long)ny * px, nz, ply, tw[1]);
-    strided(2, nz, (long long)ny * px, px, ny, plz, tw[2]);
-    strided(1, ny, px, (long long)ny * px, nz, ply, tw[1]);
-  } else {
-    strided(2, ny, px, (long long)ny * px, 1, ply, tw[1]);
+  if (e == cudaSuccess) {
+    if constexpr (sizeof(R) == 4) e = chain32(c, dev, s);
+    else e = chain64(c, s);
   }
-  k_c2r_x_exp_cnx<R, R, EPT_X, CL, 1><<<xgrid, T, xsm, s>>>(X);
-  if ((e = cudaGetLastError()) != cudaSuccess) {
+  if (e != cudaSuccess) {
     set_err("launch", cudaGetErrorString(e));
     return DGPE_ECUDA;
   }
@@ -245,8 +307,8 @@ extern "C" int dgpe_dipolar_potential_noalloc(const void *psi, void *phi, int fp
     base = g_scratch_ptr[dev];
   }
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  return fp64 ? run<double>(psi, phi, dim, n, h, kernel, qd, s, (unsigned char *)base)
-              : run<float>(psi, phi, dim, n, h, kernel, qd, s, (unsigned char *)base);
+  return fp64 ? run<double>(psi, phi, dim, n, h, kernel, qd, s, dev, (unsigned char *)base)
+              : run<float>(psi, phi, dim, n, h, kernel, qd, s, dev, (unsigned char *)base);
 }
 
 extern "C" const char *dgpe_noalloc_last_error(void) { return dgpe::g_err; }
