@@ -1499,31 +1499,56 @@ template <typename R> struct AArgs {
   double dts, gdt, gdddt, two_dt_g, two_dt_gdd;
 };
 
-template <typename R> __device__ __forceinline__ R adj_theta(const AArgs<R> &A, size_t i, cx<R> v, R *dens, R *v0) {
-  const int x = (int)(i % A.nx);
-  const size_t r = i / A.nx;
-  const int y = (int)(r % A.ny), z = (int)(r / A.ny);
-  *dens = v.x * v.x + v.y * v.y;
-  *v0 = A.vx[x] + A.vy[y] + A.vz[z];
-  return (R)A.dts * *v0 + (R)A.gdt * *dens + (R)A.gdddt * A.phi[i];
+// Four neighbouring sites of a row per thread: one set of index divisions
+// (32 bits: fewer than 2^32 sites).  A caller's state need not start on 16 bytes,
+// so the accesses are per site.  theta, the density
+// and V0 of site i0 + k, k < 4.
+template <typename R> struct AdjSites {
+  R th[4], dens[4], v0[4];
+  cx<R> v[4];
+};
+template <typename R, typename T> __device__ __forceinline__ void load4(T (&d)[4], const T *__restrict__ p) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) d[k] = p[k];
+}
+template <typename R> __device__ __forceinline__ void adj_sites(const AArgs<R> &A, unsigned i0, AdjSites<R> &s) {
+  const unsigned r = i0 / (unsigned)A.nx, x = i0 - r * (unsigned)A.nx;
+  const unsigned z = r / (unsigned)A.ny, y = r - z * (unsigned)A.ny;
+  const R vyz = A.vy[y] + A.vz[z];
+  R phi[4];
+  load4<R>(s.v, A.psi_in + i0);
+  load4<R>(phi, A.phi + i0);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    s.dens[k] = s.v[k].x * s.v[k].x + s.v[k].y * s.v[k].y;
+    s.v0[k] = A.vx[x + k] + vyz;
+    s.th[k] = (R)A.dts * s.v0[k] + (R)A.gdt * s.dens[k] + (R)A.gdddt * phi[k];
+  }
 }
 
 template <typename R>
 __global__ void k_adj_sigma(const __grid_constant__ AArgs<R> A) {
   __shared__ double red[32];
   double sn = 0.0, sv = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < A.n; i += (size_t)gridDim.x * blockDim.x) {
-    const cx<R> v = A.psi_in[i];
-    R dens, v0;
-    const R th = adj_theta(A, i, v, &dens, &v0);
-    R s, c;
-    fsincos(th, &s, &c);
-    const cx<R> ph = mk<R>(v.x * c + v.y * s, v.y * c - v.x * s);  // e^{-i th} psi
-    const cx<R> g = A.G[i];
-    const R sig = g.x * ph.y - g.y * ph.x;  // Im(conj(g) ph)
-    A.sig_out[i] = sig;
-    sn += (double)sig * dens;
-    sv += (double)sig * v0;
+  const unsigned n4 = (unsigned)(A.n / 4), gs = gridDim.x * blockDim.x;
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += gs) {
+    AdjSites<R> t;
+    adj_sites(A, 4 * i, t);
+    cx<R> g[4];
+    load4<R>(g, A.G + 4 * (size_t)i);
+    R sig[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      R s, cm1;
+      sin_cosm1<R>(t.th[k], &s, &cm1);
+      const cx<R> v = t.v[k];
+      const cx<R> ph = mk<R>(v.x + (v.x * cm1 + v.y * s), v.y + (v.y * cm1 - v.x * s));  // e^{-i th} psi
+      sig[k] = g[k].x * ph.y - g[k].y * ph.x;                                            // Im(conj(g) ph)
+      sn += (double)sig[k] * t.dens[k];
+      sv += (double)sig[k] * t.v0[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) A.sig_out[4 * (size_t)i + k] = sig[k];
   }
   sn = block_sum(sn, red);
   if (threadIdx.x == 0) A.partial[2 * blockIdx.x] = sn;
@@ -1533,31 +1558,43 @@ __global__ void k_adj_sigma(const __grid_constant__ AArgs<R> A) {
 
 template <typename R>
 __global__ void k_adj_update(const __grid_constant__ AArgs<R> A) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < A.n; i += (size_t)gridDim.x * blockDim.x) {
-    const cx<R> v = A.psi_in[i];
-    R dens, v0;
-    const R th = adj_theta(A, i, v, &dens, &v0);
-    R s, c;
-    fsincos(th, &s, &c);
-    const cx<R> g = A.G[i];
-    const R f = (R)A.two_dt_g * A.sig[i] + (R)A.two_dt_gdd * A.ksig[i];
-    // e^{+i th} G_phi + f psi_in
-    A.G[i] = mk<R>(g.x * c - g.y * s + f * v.x, g.y * c + g.x * s + f * v.y);
+  const unsigned n4 = (unsigned)(A.n / 4), gs = gridDim.x * blockDim.x;
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += gs) {
+    AdjSites<R> t;
+    adj_sites(A, 4 * i, t);
+    cx<R> g[4];
+    R sig[4], ks[4];
+    load4<R>(g, A.G + 4 * (size_t)i);
+    load4<R>(sig, A.sig + 4 * (size_t)i);
+    load4<R>(ks, A.ksig + 4 * (size_t)i);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      R s, cm1;
+      sin_cosm1<R>(t.th[k], &s, &cm1);
+      const R f = (R)A.two_dt_g * sig[k] + (R)A.two_dt_gdd * ks[k];
+      // e^{+i th} G_phi + f psi_in
+      g[k] = mk<R>(g[k].x + (g[k].x * cm1 - g[k].y * s) + f * t.v[k].x, g[k].y + (g[k].y * cm1 + g[k].x * s) + f * t.v[k].y);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) A.G[4 * (size_t)i + k] = g[k];
   }
 }
 
 // Fixed-order totals of the per-block partials, accumulated in FP64:
-// acc[0] += dt S_n,  acc[1 + m - 1] += dt sin(m t) S_V.
+// acc[0] += dt S_n,  acc[1 + m - 1] += dt sin(m t) S_V (one thread per m).
 static __global__ void k_adj_accumulate(const double *partial, int nblk, double *acc, double dt, double t, int M) {
-  __shared__ double red[32];
+  __shared__ double red[32], s_b;
   double a = 0.0, b = 0.0;
+  const double w = threadIdx.x >= 1 && (int)threadIdx.x <= M ? dt * sin((double)threadIdx.x * t) : 0.0;
   for (int i = threadIdx.x; i < nblk; i += blockDim.x) { a += partial[2 * i]; b += partial[2 * i + 1]; }
   a = block_sum(a, red);
   b = block_sum(b, red);
   if (threadIdx.x == 0) {
     acc[0] += dt * a;
-    for (int m = 1; m <= M; ++m) acc[m] += dt * sin((double)m * t) * b;
+    s_b = b;
   }
+  __syncthreads();
+  if (threadIdx.x >= 1 && (int)threadIdx.x <= M) acc[threadIdx.x] += w * s_b;
 }
 
 // partial[block] = sum conj(a) b (complex, FP64)
