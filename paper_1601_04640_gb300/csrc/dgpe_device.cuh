@@ -80,8 +80,6 @@ static __device__ __noinline__ double2 sincos_call(double a) { double2 r; sincos
 static __device__ __noinline__ float2 sincos_call(float a) { float2 r; sincosf(a, &r.x, &r.y); return r; }
 static __device__ __noinline__ double expm1_call(double a) { return expm1(a); }
 static __device__ __noinline__ float expm1_call(float a) { return expm1f(a); }
-__device__ __forceinline__ void fsincos(double a, double *s, double *c) { sincos(a, s, c); }
-__device__ __forceinline__ void fsincos(float a, float *s, float *c) { sincosf(a, s, c); }
 // expm1: for |a| <= 1/8 its Taylor series a + a^2 (1/2! + a/3! + ...) through
 // a^10 / 10! in FP64 and a^6 / 6! in FP32 (first omitted terms 2.3e-17 and
 // 7.6e-10 relative at 1/8), which is 10 and 6 multiply-adds; beyond that the

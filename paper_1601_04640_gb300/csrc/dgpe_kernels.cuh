@@ -1502,56 +1502,33 @@ template <typename R> struct AArgs {
   double dts, gdt, gdddt, two_dt_g, two_dt_gdd;
 };
 
-// Four neighbouring sites of a row per thread: one set of index divisions
-// (32 bits: fewer than 2^32 sites).  A caller's state need not start on 16 bytes,
-// so the accesses are per site.  theta, the density
-// and V0 of site i0 + k, k < 4.
-template <typename R> struct AdjSites {
-  R th[4], dens[4], v0[4];
-  cx<R> v[4];
-};
-template <typename R, typename T> __device__ __forceinline__ void load4(T (&d)[4], const T *__restrict__ p) {
-#pragma unroll
-  for (int k = 0; k < 4; ++k) d[k] = p[k];
-}
-template <typename R> __device__ __forceinline__ void adj_sites(const AArgs<R> &A, unsigned i0, AdjSites<R> &s) {
-  const unsigned r = i0 / (unsigned)A.nx, x = i0 - r * (unsigned)A.nx;
+// theta, the density and V0 of site i (32-bit divisions: fewer than 2^32
+// sites; 64-bit ones and the library's sincos at every site were most of these
+// kernels, 24 us each at 128^3).
+template <typename R> __device__ __forceinline__ R adj_theta(const AArgs<R> &A, unsigned i, cx<R> v, R *dens, R *v0) {
+  const unsigned r = i / (unsigned)A.nx, x = i - r * (unsigned)A.nx;
   const unsigned z = r / (unsigned)A.ny, y = r - z * (unsigned)A.ny;
-  const R vyz = A.vy[y] + A.vz[z];
-  R phi[4];
-  load4<R>(s.v, A.psi_in + i0);
-  load4<R>(phi, A.phi + i0);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    s.dens[k] = s.v[k].x * s.v[k].x + s.v[k].y * s.v[k].y;
-    s.v0[k] = A.vx[x + k] + vyz;
-    s.th[k] = (R)A.dts * s.v0[k] + (R)A.gdt * s.dens[k] + (R)A.gdddt * phi[k];
-  }
+  *dens = v.x * v.x + v.y * v.y;
+  *v0 = A.vx[x] + A.vy[y] + A.vz[z];
+  return (R)A.dts * *v0 + (R)A.gdt * *dens + (R)A.gdddt * A.phi[i];
 }
 
 template <typename R>
 __global__ void k_adj_sigma(const __grid_constant__ AArgs<R> A) {
   __shared__ double red[32];
   double sn = 0.0, sv = 0.0;
-  const unsigned n4 = (unsigned)(A.n / 4), gs = gridDim.x * blockDim.x;
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += gs) {
-    AdjSites<R> t;
-    adj_sites(A, 4 * i, t);
-    cx<R> g[4];
-    load4<R>(g, A.G + 4 * (size_t)i);
-    R sig[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      R s, cm1;
-      sin_cosm1<R>(t.th[k], &s, &cm1);
-      const cx<R> v = t.v[k];
-      const cx<R> ph = mk<R>(v.x + (v.x * cm1 + v.y * s), v.y + (v.y * cm1 - v.x * s));  // e^{-i th} psi
-      sig[k] = g[k].x * ph.y - g[k].y * ph.x;                                            // Im(conj(g) ph)
-      sn += (double)sig[k] * t.dens[k];
-      sv += (double)sig[k] * t.v0[k];
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) A.sig_out[4 * (size_t)i + k] = sig[k];
+  const unsigned n = (unsigned)A.n, gs = gridDim.x * blockDim.x;
+#pragma unroll 2
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gs) {
+    const cx<R> v = A.psi_in[i], g = A.G[i];
+    R dens, v0, s, cm1;
+    const R th = adj_theta(A, i, v, &dens, &v0);
+    sin_cosm1<R>(th, &s, &cm1);
+    const cx<R> ph = mk<R>(v.x + (v.x * cm1 + v.y * s), v.y + (v.y * cm1 - v.x * s));  // e^{-i th} psi
+    const R sig = g.x * ph.y - g.y * ph.x;                                             // Im(conj(g) ph)
+    A.sig_out[i] = sig;
+    sn += (double)sig * dens;
+    sv += (double)sig * v0;
   }
   sn = block_sum(sn, red);
   if (threadIdx.x == 0) A.partial[2 * blockIdx.x] = sn;
@@ -1561,25 +1538,16 @@ __global__ void k_adj_sigma(const __grid_constant__ AArgs<R> A) {
 
 template <typename R>
 __global__ void k_adj_update(const __grid_constant__ AArgs<R> A) {
-  const unsigned n4 = (unsigned)(A.n / 4), gs = gridDim.x * blockDim.x;
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += gs) {
-    AdjSites<R> t;
-    adj_sites(A, 4 * i, t);
-    cx<R> g[4];
-    R sig[4], ks[4];
-    load4<R>(g, A.G + 4 * (size_t)i);
-    load4<R>(sig, A.sig + 4 * (size_t)i);
-    load4<R>(ks, A.ksig + 4 * (size_t)i);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      R s, cm1;
-      sin_cosm1<R>(t.th[k], &s, &cm1);
-      const R f = (R)A.two_dt_g * sig[k] + (R)A.two_dt_gdd * ks[k];
-      // e^{+i th} G_phi + f psi_in
-      g[k] = mk<R>(g[k].x + (g[k].x * cm1 - g[k].y * s) + f * t.v[k].x, g[k].y + (g[k].y * cm1 + g[k].x * s) + f * t.v[k].y);
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) A.G[4 * (size_t)i + k] = g[k];
+  const unsigned n = (unsigned)A.n, gs = gridDim.x * blockDim.x;
+#pragma unroll 2
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gs) {
+    const cx<R> v = A.psi_in[i], g = A.G[i];
+    R dens, v0, s, cm1;
+    const R th = adj_theta(A, i, v, &dens, &v0);
+    sin_cosm1<R>(th, &s, &cm1);
+    const R f = (R)A.two_dt_g * A.sig[i] + (R)A.two_dt_gdd * A.ksig[i];
+    // e^{+i th} G_phi + f psi_in
+    A.G[i] = mk<R>(g.x + (g.x * cm1 - g.y * s) + f * v.x, g.y + (g.y * cm1 + g.x * s) + f * v.y);
   }
 }
 

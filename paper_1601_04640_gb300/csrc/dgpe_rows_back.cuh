@@ -34,7 +34,7 @@ __device__ __forceinline__ float2 phase_update(float2 v, float sn, float cm1) { 
 template <int CL> __device__ __forceinline__ void exp_real_time(float2 (&v)[CL], const float (&th)[CL]) {
   float m = 0.0f;
 #pragma unroll
-  for (int i = 0; i < CL; ++i) m = fabsf(th[i]) <= m ? m : fabsf(th[i]);  // a NaN stays
+  for (int i = 0; i < CL; ++i) m = fabsf(th[i]) <= m ? m : fabsf(th[i]);  // a NaN gives NaN on any path
   if (m <= 0.125f) {
 #pragma unroll
     for (int i = 0; i < CL; ++i) {
