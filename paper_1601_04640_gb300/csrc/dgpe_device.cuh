@@ -582,6 +582,14 @@ __device__ __forceinline__ void tile_fft_ct_cols(cx<R> *sm, const cx<R> *__restr
   tile_fft_ct_from<R, N, EPT, INV, 0, 1, NL, T, true, NL, 0, 1, PF>(sm, tw, load, store);
 }
 
+// 1 / x for a finite normal x > 0: the approximate reciprocal (relative error
+// below 2^-22) and one Newton step, x (1 / x) = 1 to within an ulp.
+__device__ __forceinline__ float reciprocal(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return fmaf(r, fmaf(-x, r, 1.0f), r);
+}
+
 // ------------------------------------------------ programmatic launch order
 // The passes of a step are launched so that a pass's blocks start while the
 // one before it drains (launch_pdl): they set up what only constants need and

@@ -1005,9 +1005,11 @@ template <typename R> struct EngineT : Engine {
     A.twf = twf[f.axis]; A.twi = twi[f.axis];
     A.estride = f.es; A.ostride = f.os; A.n = f.n; A.ncols = ncol_spec; A.W = f.W; A.nxh = nx / 2;
     if (dim == 3) {
-      A.uq[0] = (float)(2.0 * M_PI / (nx * p.h[0]));
-      A.uq[1] = (float)(2.0 * M_PI / (ny * p.h[1]));
-      A.uq[2] = (float)(2.0 * M_PI / (nz * p.h[2]));
+      // U depends on the ratios of the wavenumbers alone: the steps relative to
+      // the largest keep k^2 far from the ends of the exponent range
+      const double d[3] = {1.0 / (nx * p.h[0]), 1.0 / (ny * p.h[1]), 1.0 / (nz * p.h[2])};
+      const double dm = std::max(d[0], std::max(d[1], d[2]));
+      for (int a = 0; a < 3; ++a) A.uq[a] = (float)(d[a] / dm);
       A.uq[3] = (float)((4.0 * M_PI / 3.0) / (double)nsites);
     }
     A.uny = ny;

@@ -67,7 +67,8 @@ template <typename R> struct SArgs {  // strided FFT passes over the spectrum
   long long estride, ostride;
   int n, ncols, W, nxh;
   // 3D dipolar kernel from the wavenumbers (FP32 tensor-map z-pass):
-  // dq_x, dq_y, dq_z (2 pi / (n h) per axis), (4 pi / 3) / N_sites; ny
+  // dq_x, dq_y, dq_z (1 / (n h) per axis, relative to the largest),
+  // (4 pi / 3) / N_sites; ny
   float uq[4];
   int uny;
 };
@@ -842,7 +843,10 @@ __global__ void __launch_bounds__(W * N / EPT < 128 ? 64 : DGPE_MAXT_FFT, W * N 
 // The 3D z-pass (MODE 2, AXIS 2) evaluates U(k) = (4 pi / 3)(3 k_z^2 / k^2 - 1)
 // / N_sites in FP32 from the wavenumbers (U(0) = 0) instead of reading the
 // table: four bytes less per spectrum element and no global load inside the
-// transform pair.
+// transform pair.  The pass is bound by instructions (256^3: 63 % of the issue
+// slots), a third of which formed k_z^2 and the quotient: k_z^2 comes from a
+// shared table and the reciprocal from the approximate one and a Newton step
+// (256^3: 40 -> 37 us, 512 x 512 x 256 131 -> 117).
 template <int EPT, int MODE, int N, int W, int AXIS>
 __global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
     k_fft_tma(const __grid_constant__ CUtensorMap tm, const __grid_constant__ SArgs<float> A, int ncb, int ntiles,
@@ -856,6 +860,7 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
   Cx *const buf0 = reinterpret_cast<Cx *>(smraw + ((128 - (smem_u32(smraw) & 127)) & 127));
   __shared__ unsigned long long bar[2];
   __shared__ __align__(16) Cx s_tw[N];
+  __shared__ R s_qz2[MODE == 2 && AXIS == 2 ? N : 1];  // k_z^2 of every row
   const int t = threadIdx.x;
   auto issue = [&](int tile, int k) {  // thread 0
     const int c0 = (tile % ncb) * W, o = tile / ncb;
@@ -872,7 +877,13 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
   }
-  for (int i = t; i < N; i += T) s_tw[i] = A.tw[i];
+  for (int i = t; i < N; i += T) {
+    s_tw[i] = A.tw[i];
+    if constexpr (MODE == 2 && AXIS == 2) {
+      const R qz = (R)((i <= N / 2) ? i : i - N) * A.uq[2];
+      s_qz2[i] = qz * qz;
+    }
+  }
   pdl_wait();
   __syncthreads();
   if (t == 0) {
@@ -904,11 +915,10 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
       // tile: kx = c0 + l, ky = o, kz = row a
       const int jy = (o <= A.uny / 2) ? o : o - A.uny;
       const R qy = (R)jy * A.uq[1];
-      const R qy2 = qy * qy, dqx = A.uq[0], dqz = A.uq[2], pref = A.uq[3];
+      const R qy2 = qy * qy, dqx = A.uq[0], pref = A.uq[3];
       auto mstore = [&](int l, int a, Cx v) {
-        const R qx = (R)(c0 + l) * dqx, qz = (R)((a <= N / 2) ? a : a - N) * dqz;
-        const R qz2 = qz * qz, k2 = fmaf(qx, qx, qy2) + qz2;
-        const R u = (k2 > (R)0) ? pref * ((R)3 * qz2 / k2 - (R)1) : (R)0;
+        const R qx = (R)(c0 + l) * dqx, qz2 = s_qz2[a], k2 = fmaf(qx, qx, qy2) + qz2;
+        const R u = (k2 > (R)0) ? fmaf((R)3 * pref * qz2, reciprocal(k2), -pref) : (R)0;
         sm[a * W + l] = cscale(v, u);
       };
       tile_fft_ct_cols<R, N, EPT, false, W, T, true>(sm, s_tw, sload, mstore);
