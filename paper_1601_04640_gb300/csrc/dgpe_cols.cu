@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(kColsThreads, 3)
   const int a0 = q * CL;
   double acc = 0.0;
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const unsigned c = ((unsigned)tile << lw) + (unsigned)lc;
+    const unsigned c = ((unsigned)(A.back ? ntiles - 1 - tile : tile) << lw) + (unsigned)lc;
     const bool ok = c < A.tot;
     const unsigned o = c / A.ncols;
     float2 *const p = A.psi + (size_t)o * A.os + (c - o * A.ncols) + (size_t)a0 * A.es;

@@ -862,8 +862,11 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
   __shared__ __align__(16) Cx s_tw[N];
   __shared__ R s_qz2[MODE == 2 && AXIS == 2 ? N : 1];  // k_z^2 of every row
   const int t = threadIdx.x;
+  // the inverse transform runs from the last plane to the first: the x pass
+  // behind it starts with the first
+  auto at = [&](int tile) { return MODE == 1 ? ntiles - 1 - tile : tile; };
   auto issue = [&](int tile, int k) {  // thread 0
-    const int c0 = (tile % ncb) * W, o = tile / ncb;
+    const int c0 = (at(tile) % ncb) * W, o = at(tile) / ncb;
     Cx *dst = buf0 + k * TILE;
     fence_proxy_async_smem();
     mbar_expect_tx(&bar[k], (unsigned)(sizeof(Cx) * TILE));
@@ -904,7 +907,7 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
       return;
     }
     Cx *const sm = buf0 + k * TILE;
-    const int c0 = (tile % ncb) * W, o = tile / ncb;
+    const int c0 = (at(tile) % ncb) * W, o = at(tile) / ncb;
     auto sload = [&](int l, int a) -> Cx { return sm[a * W + l]; };
     auto sstore = [&](int l, int a, Cx v) { sm[a * W + l] = v; };
     if constexpr (MODE == 0) {

@@ -50,6 +50,7 @@ struct ColArgs {
   long long es, os;
   unsigned tot, ncols;
   int n, cl;       // points; points per chunk (16, 12 or 10)
+  int back;        // tiles from the last to the first
   int nsm;         // SMs, as in cols_grid
   int final_pass, norm;
   int early;       // launch_pdl
