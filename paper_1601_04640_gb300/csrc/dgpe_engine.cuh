@@ -334,6 +334,7 @@ template <typename R> struct EngineT : Engine {
   // real state (imaginary time): psi holds nx reals per row, viewed by the
   // strided CN passes as nx/2 complex columns (pairs of real lines)
   bool rpsi = false;
+  Cx *ocx = nullptr;  // complex copy of a real state for the observables
 
   ~EngineT() override {
     if (gexec) cudaGraphExecDestroy(gexec);
@@ -342,7 +343,7 @@ template <typename R> struct EngineT : Engine {
     void *bufs[] = {psi, spec, U, phi_tmp, tw[0], tw[1], tw[2], vt[0], vt[1], vt[2],
                     cntab[0], cntab[1], cntab[2], prm, partial, obs_part, dip_part, obs_out,
                     dstep, counter, stage, adjG, adjT, adj_phi, adj_sig, adj_ksig, adj_part,
-                    adj_acc, cntab_adj[0], cntab_adj[1], cntab_adj[2], fineE, twf[0], twf[1], twf[2],
+                    adj_acc, cntab_adj[0], cntab_adj[1], cntab_adj[2], fineE, ocx, twf[0], twf[1], twf[2],
                     twi[0], twi[1], twi[2]};
     for (void *b : bufs)
       if (b) cudaFree(b);
@@ -1638,8 +1639,18 @@ template <typename R> struct EngineT : Engine {
   int observables(dgpe_obs *o, cudaStream_t s) override {
     int rc;
     DGPE_LCK("(pending before observables)");
+    // a real state is widened to (psi, 0) first; the sums below then run
+    // unchanged on the complex copy
+    const Cx *obs_psi = psi;
+    if (rpsi) {
+      if (!ocx && (rc = dalloc(&ocx, nsites))) return rc;
+      k_widen_real<R><<<152 * 8, 256, 0, s>>>(ocx, (const R *)psi, nsites);
+      launched(1);
+      DGPE_LCK("widen");
+      obs_psi = ocx;
+    }
     if (has_dip) {
-      if ((rc = launch_forward_spectrum(s))) return rc;
+      if ((rc = launch_forward_spectrum(s, obs_psi))) return rc;
       DGPE_LCK("density/R2C");
       if (dim == 3) {
         if ((rc = launch_fft(fy, 0, s))) return rc;
@@ -1650,11 +1661,10 @@ template <typename R> struct EngineT : Engine {
       DGPE_LCK("spectral energy sum");
     }
     OArgs<R> A{};
-    A.psi = psi; A.prm = prm; A.partial = obs_part; A.nx = nx; A.ny = ny; A.nz = nz; A.dim = dim;
+    A.psi = obs_psi; A.prm = prm; A.partial = obs_part; A.nx = nx; A.ny = ny; A.nz = nz; A.dim = dim;
     A.rows = obs_rows; A.hx = p.h[0]; A.hy = p.h[1]; A.hz = (dim == 3) ? p.h[2] : 0.0;
     A.nux = p.nu[0]; A.nuy = p.nu[1]; A.nuz = (dim == 3) ? p.nu[2] : 0.0;
-    if (rpsi) k_obs_sites<R, true><<<obs_blocks, 256, 0, s>>>(A);
-    else k_obs_sites<R, false><<<obs_blocks, 256, 0, s>>>(A);
+    k_obs_sites<R><<<obs_blocks, 256, 0, s>>>(A);
     launched(1);
     DGPE_LCK("site sums");
     k_obs_final<<<OBS_COUNT + 1, 256, 0, s>>>(obs_part, obs_blocks, dip_part, ndip, prm, dstep, obs_out);

@@ -1375,19 +1375,18 @@ __global__ void __launch_bounds__(128) k_cn_lines(const __grid_constant__ LArgs 
 enum { OBS_N, OBS_X2, OBS_Y2, OBS_Z2, OBS_V, OBS_N2, OBS_KX, OBS_KY, OBS_KZ, OBS_BAD, OBS_COUNT };
 
 // Four neighbouring sites of a row per thread, walked along y with the row
-// above kept, over A.rows rows of one z.  REAL: psi holds nx reals per row.
+// above kept, over A.rows rows of one z.
 //
 // Bound by FP64 instructions (64 cycles per warp and scheduler), so what a sum
 // shares is taken out of the sites: the state is converted once per site and
 // once for its z neighbour, y^2 and z^2 multiply the row's sum, V0 is formed
 // from the moments and (FP32, whose n^2 cannot overflow in FP64) the scale is
-// applied to the sums: 22 instead of 66 per site, 13 for a real state.  All
-// observables of 256^3: 1.98 -> 1.26 ms, with a real state 2.21 -> 0.83 ms; of
-// 512 x 512 x 256 7.5 -> 4.3 ms.
-template <typename R, bool REAL>
+// applied to the sums: 22 instead of 66 per site.  All observables of
+// 256^3: 1.98 -> 1.26 ms, of 512 x 512 x 256 7.5 -> 4.3 ms.
+template <typename R>
 __global__ void __launch_bounds__(256) k_obs_sites(const __grid_constant__ OArgs<R> A) {
   __shared__ double red[32];
-  constexpr int NC = REAL ? 1 : 2, V = 4;  // components, sites per thread
+  constexpr int NC = 2, V = 4;  // components, sites per thread
   constexpr bool SCALED = sizeof(R) == 8;
   const int nx = A.nx, ny = A.ny, nz = A.nz;
   const R *const psi = reinterpret_cast<const R *>(A.psi);
@@ -1642,6 +1641,12 @@ __global__ void k_export_real(S *dst, const R *src, const double *prm, size_t n)
     o.y = (decltype(o.y))0;
     dst[i] = o;
   }
+}
+// real state -> complex (v, 0), unscaled (the observables' input)
+template <typename R>
+__global__ void k_widen_real(cx<R> *dst, const R *src, size_t n) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+    dst[i] = mk<R>(src[i], (R)0);
 }
 template <typename R>
 __global__ void k_fold_scale(cx<R> *psi, double *prm, size_t n) {
