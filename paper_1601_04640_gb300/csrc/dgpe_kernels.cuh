@@ -921,7 +921,8 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
       const R qy2 = qy * qy, dqx = A.uq[0], pref = A.uq[3];
       auto mstore = [&](int l, int a, Cx v) {
         const R qx = (R)(c0 + l) * dqx, qz2 = s_qz2[a], k2 = fmaf(qx, qx, qy2) + qz2;
-        const R u = (k2 > (R)0) ? fmaf((R)3 * pref * qz2, reciprocal(k2), -pref) : (R)0;
+        // 3 k_z^2 / k^2 first: a rounded 3 pref would shift the mean of U
+        const R u = (k2 > (R)0) ? fmaf(pref, (R)3 * qz2 * reciprocal(k2), -pref) : (R)0;
         sm[a * W + l] = cscale(v, u);
       };
       tile_fft_ct_cols<R, N, EPT, false, W, T, true>(sm, s_tw, sload, mstore);

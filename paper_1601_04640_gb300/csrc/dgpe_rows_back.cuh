@@ -26,7 +26,7 @@ template <int CL, bool REAL> struct RowStage {
 
 // The exponential of a lane's CL sites.  A lane whose exponents all lie within
 // 1/8 takes the short Taylor series (sin_cosm1, fexpm1), within 2 (1) the
-// series below, whose first omitted terms are below 2e-10 (3e-8) relative;
+// series below, whose first omitted terms are below 2e-10 (3e-9) relative;
 // beyond that the library functions, out of line.
 __device__ __forceinline__ float2 phase_update(float2 v, float sn, float cm1) {  // v e^{-i th}, as in nonlinear_factor
   return make_float2(v.x + (v.x * cm1 + v.y * sn), v.y + (v.y * cm1 - v.x * sn));
@@ -90,7 +90,8 @@ template <int CL> __device__ __forceinline__ void exp_imag_time(float (&th)[CL])
 #pragma unroll
     for (int i = 0; i < CL; ++i) {
       const float a = -th[i];
-      float p = 1.0f / 3628800.0f;
+      float p = 1.0f / 39916800.0f;
+      p = fmaf(p, a, 1.0f / 3628800.0f);
       p = fmaf(p, a, 1.0f / 362880.0f);
       p = fmaf(p, a, 1.0f / 40320.0f);
       p = fmaf(p, a, 1.0f / 5040.0f);
