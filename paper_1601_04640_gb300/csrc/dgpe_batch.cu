@@ -17,7 +17,6 @@
 
 #include "dgpe.h"
 #include "dgpe_engine.cuh"
-#include "dgpe_rows_back.cuh"
 
 namespace dgpe {
 namespace {
@@ -63,11 +62,7 @@ struct BProb {
   int var, imag, resident, n;
   int tiles[4];  // per pass of one step
   int per_step;  // tiles of one step
-  // constant-coefficient forms along x and y (dgpe_lines.cuh) and whether they
-  // are taken (rows: in x, cols: in y; otherwise the table forms)
-  int rows, cols;
-  CnConst<float> kxr, kyr;
-  CnConst<float2> kxc, kyc;
+  int pad[3];
 };
 // work-list state in device memory (unsigned words): the ticket counter, CTAs
 // that have left, the abort and timeout flags, the held problem + 1 (0: none),
@@ -265,188 +260,14 @@ __device__ __forceinline__ void batch_pass(const BProb &B, int level, int tile) 
   switch (level) {
     case 0: batch_body<EX, EPS, CL, P2, N, 0, float>(B, tile); break;
     case 1: batch_body<EX, EPS, CL, P2, N, 1, float>(B, tile); break;
-    // the table forms (slowly decaying coefficients; batch_lines has the others)
     case 2:
-      if (B.imag) batch_body<EX, EPS, CL, P2, 0, 2, float>(B, tile);
-      else batch_body<EX, EPS, CL, P2, 0, 2, float2>(B, tile);
+      if (B.imag) batch_body<EX, EPS, CL, P2, N, 2, float>(B, tile);
+      else batch_body<EX, EPS, CL, P2, N, 2, float2>(B, tile);
       break;
     default:
-      if (B.imag) batch_body<EX, EPS, CL, P2, 0, 3, float>(B, tile);
-      else batch_body<EX, EPS, CL, P2, 0, 3, float2>(B, tile);
+      if (B.imag) batch_body<EX, EPS, CL, P2, N, 3, float>(B, tile);
+      else batch_body<EX, EPS, CL, P2, N, 3, float2>(B, tile);
   }
-}
-// C2R_x, exponential and CN_x of eight warp tiles (dgpe_rows_back.cuh).  There
-// is no tensor map per problem: a warp copies its rows with cp.async, the second
-// row of each pair into the transform's lines once Phi_d has left them.
-constexpr int kRowWarpsBatch = DGPE_MAXT / 32;
-template <int N> constexpr int batch_rows_smem() { return kRowWarpsBatch * (32 * Row<N>::CL + Row<N>::ZEL + 1) * 8; }
-template <int N, typename Coef>
-__device__ __noinline__ void batch_rows(const XArgs<float> &X, const CnConst<Coef> &K, int tile) {
-  typedef Row<N> C;
-  typedef RowStage<C::CL, false> G;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int CL = C::CL, TPL = C::TPL, NL = C::NL, SE = 32 * CL, ZE = (C::ZEL + 1) & ~1, PC = N / 2;  // pieces per row
-  constexpr bool RT = std::is_same<Coef, float2>::value;
-  constexpr int OFF_VX = 8 * N, OFF_K = OFF_VX + 4 * N;
-  static_assert(OFF_K + 16 <= kBatchScr && ZE >= NL * N, "shared scratch");
-  unsigned char *const scr = shared_scratch<kBatchScr>();
-  float2 *const tws = reinterpret_cast<float2 *>(scr);
-  float4 *const vxs = reinterpret_cast<float4 *>(scr + OFF_VX);
-  float *const s_k = reinterpret_cast<float *>(scr + OFF_K);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane / TPL, q = lane % TPL;
-  unsigned char *const st = smraw + w * SE * 8;
-  float2 *const z = reinterpret_cast<float2 *>(smraw + kRowWarpsBatch * SE * 8) + w * ZE;
-  const int row0 = (tile * kRowWarpsBatch + w) * C::ROWS;
-  // 16-byte piece k of the tile's rows of parity h: chunk k / NP, piece k % NP
-  auto fetch = [&](unsigned char *dst, int h) {
-#pragma unroll
-    for (int k = 0; k < G::NP; ++k) {
-      const unsigned p = lane + 32 * k, ll = p / PC, o = p % PC;
-      const int row = row0 + 2 * (int)ll + h;
-      if (row < X.nrows) cp_async16(dst + G::off(p / G::NP, p % G::NP), X.psi + (size_t)row * N + 2 * o);
-    }
-    cp_async_commit();
-  };
-  fetch(st, 0);
-  if (X.has_dip)
-    for (int p = lane; p < C::ROWS * (C::PX / 2); p += 32) {
-      const int r = p / (C::PX / 2), o = p % (C::PX / 2);
-      if (row0 + r < X.nrows)
-        cp_async16(z + ((r >> 1) + (r & 1) * NL) * C::PS + 2 * o, X.spec + (size_t)(row0 + r) * C::PX + 2 * o);
-    }
-  cp_async_commit();
-  row_twiddles<N>(tws, X.tw);
-  for (int i = threadIdx.x; i < N; i += blockDim.x)
-    reinterpret_cast<float *>(vxs)[((i % CL) / 4 * TPL + i / CL) * 4 + i % 4] = X.vx[i];
-  if (threadIdx.x == 0) {
-    s_k[0] = (float)(trap_dts(X.prm, *X.step) * X.dtf);
-    s_k[1] = (float)(X.prm[PRM_DT] * X.dtf * X.prm[PRM_G]);
-    s_k[2] = (float)(X.prm[PRM_DT] * X.dtf * X.prm[PRM_GDD]);
-    s_k[3] = (float)X.prm[PRM_SC];
-  }
-  cp_async_wait<0>();
-  __syncthreads();
-  if (row0 >= X.nrows) return;
-  const float dts = s_k[0], gdt = s_k[1], gdddt = s_k[2], sc = RT ? 1.0f : s_k[3];
-  float2 f[CL];
-  if (X.has_dip) {
-    row_c2r<N>(z, z + l * C::PS, z + (l + NL) * C::PS, q);
-    row_stages<N, CL, 0, true>(z, tws);
-  }
-#pragma unroll
-  for (int i = 0; i < CL; ++i) f[i] = X.has_dip ? z[l * C::SL + q * (CL + 1) + i] : make_float2(0.0f, 0.0f);
-  __syncwarp();
-  unsigned char *buf = st;
-  fetch(reinterpret_cast<unsigned char *>(z), 1);
-#pragma unroll 1
-  for (int h = 0; h < 2; ++h) {
-    if (h) {
-      cp_async_wait<0>();
-      __syncwarp();
-      buf = reinterpret_cast<unsigned char *>(z);
-    }
-    float2 v[CL];
-#pragma unroll
-    for (int c = 0; c < G::NP; ++c) {
-      const float4 a = *reinterpret_cast<const float4 *>(buf + G::off(lane, c));
-      v[2 * c] = make_float2(a.x, a.y);
-      v[2 * c + 1] = make_float2(a.z, a.w);
-    }
-    const int row = min(row0 + 2 * l + h, X.nrows - 1);
-    const float vr = X.vy[row % X.ny] + X.vz[row / X.ny];
-    float th[CL];
-#pragma unroll
-    for (int c = 0; c < CL / 4; ++c) {
-      const float4 x4 = vxs[c * TPL + q];
-      const float xs[4] = {x4.x, x4.y, x4.z, x4.w};
-#pragma unroll
-      for (int i = 4 * c; i < 4 * c + 4; ++i) {
-        if (!RT) v[i] = cscale(v[i], sc);
-        th[i] = dts * (xs[i - 4 * c] + vr) + gdt * (v[i].x * v[i].x + v[i].y * v[i].y) + gdddt * f[i].x;
-        f[i].x = f[i].y;  // the second row's Phi_d
-      }
-    }
-    if constexpr (RT) {
-      exp_real_time<CL>(v, th);
-    } else {
-      exp_imag_time<CL>(th);
-#pragma unroll
-      for (int i = 0; i < CL; ++i) v[i] = make_float2(v[i].x + v[i].x * th[i], v[i].y + v[i].y * th[i]);
-    }
-    row_solve<Coef, CL, TPL>(v, q, K);
-#pragma unroll
-    for (int c = 0; c < G::NP; ++c)
-      *reinterpret_cast<float4 *>(buf + G::off(lane, c)) = make_float4(v[2 * c].x, v[2 * c].y, v[2 * c + 1].x, v[2 * c + 1].y);
-    __syncwarp();
-#pragma unroll
-    for (int k = 0; k < G::NP; ++k) {
-      const unsigned p = lane + 32 * k, ll = p / PC, o = p % PC;
-      const int r = row0 + 2 * (int)ll + h;
-      if (r < X.nrows)
-        *reinterpret_cast<float4 *>(X.psi + (size_t)r * N + 2 * o) =
-            *reinterpret_cast<const float4 *>(buf + G::off(p / G::NP, p % G::NP));
-    }
-  }
-}
-template <int N> __device__ __forceinline__ void batch_rows(const BProb &B, int tile) {
-  if (B.imag) batch_rows<N, float>(B.X, B.kxr, tile);
-  else batch_rows<N, float2>(B.X, B.kxc, tile);
-}
-// CN_y (+ norm) of W columns, as in dgpe_cols.cu
-template <typename Coef, int CL>
-__device__ __noinline__ void batch_cols(const CArgs<float> &A, const CnConst<Coef> &K, int tile, int ntiles) {
-  constexpr int OFF_LAST = scr_align(sizeof(double) * 32), OFF_SE = OFF_LAST + 32;
-  static_assert(OFF_SE + 2 * DGPE_MAXT * 8 <= kBatchScr, "shared scratch");
-  unsigned char *const scr = shared_scratch<kBatchScr>();
-  float2 *const se = reinterpret_cast<float2 *>(scr + OFF_SE);
-  const int lw = ilog2(A.W), t = threadIdx.x, lc = t & (A.W - 1), q = t >> lw, tpl = A.n / CL;
-  const int c = tile * A.W + lc;
-  const bool ok = c < A.ncols && q < tpl;
-  float2 *const p = A.psi + c + (size_t)(q * CL) * A.estride;
-  float2 v[CL], y[CL], prev = make_float2(0.0f, 0.0f), next = prev;
-#pragma unroll
-  for (int i = 0; i < CL; ++i) v[i] = prev;
-  if (ok) {
-    if (q > 0) prev = *(p - A.estride);
-#pragma unroll
-    for (int i = 0; i < CL; ++i) v[i] = p[(size_t)i * A.estride];
-    if (q < tpl - 1) next = p[(size_t)CL * A.estride];
-  }
-  col_solve<Coef, CL>(v, y, prev, next, q, tpl, lw, lc, se, K);
-  double acc = 0.0;
-  if (ok) {
-    float ts = 0.0f;
-#pragma unroll
-    for (int i = 0; i < CL; ++i) {
-      p[(size_t)i * A.estride] = v[i];
-      ts += v[i].x * v[i].x + v[i].y * v[i].y;
-    }
-    acc = (double)ts;
-  }
-  cn_final(A, acc, (unsigned)ntiles, (unsigned)tile, reinterpret_cast<double *>(scr),
-           *reinterpret_cast<int *>(scr + OFF_LAST));
-}
-template <int CL> __device__ __forceinline__ void batch_cols(const BProb &B, int tile) {
-  if (B.imag) batch_cols<float, CL>(B.C, B.kyr, tile, B.tiles[3]);
-  else batch_cols<float2, CL>(B.C, B.kyc, tile, B.tiles[3]);
-}
-// passes 2 and 3 in the constant-coefficient form; false: the table form
-__device__ __forceinline__ bool batch_lines(const BProb &B, int level, int tile) {
-  if (level == 3 && B.cols) {
-    if (B.var == VAR_P2) batch_cols<16>(B, tile);
-    else if (B.var == VAR_3) batch_cols<12>(B, tile);
-    else batch_cols<10>(B, tile);
-    return true;
-  }
-  if (level != 2 || !B.rows) return false;
-  switch (B.n) {
-#define DGPE_ROW(N) case N: batch_rows<N>(B, tile); return true;
-    DGPE_ROW(32) DGPE_ROW(64) DGPE_ROW(128) DGPE_ROW(256) DGPE_ROW(512)
-    DGPE_ROW(48) DGPE_ROW(96) DGPE_ROW(192) DGPE_ROW(384)
-    DGPE_ROW(40) DGPE_ROW(80) DGPE_ROW(160) DGPE_ROW(320)
-#undef DGPE_ROW
-  }
-  return false;
 }
 template <typename Coef>
 __device__ __noinline__ void batch_resident(const BProb &B, int nsteps) {
@@ -515,7 +336,6 @@ __global__ void __launch_bounds__(DGPE_MAXT, 2)
       if (level == 4) {
         if (B.imag) batch_resident<float>(B, nsteps);
         else batch_resident<float2>(B, nsteps);
-      } else if (batch_lines(B, level, tile)) {
       } else if (B.var == VAR_P2 && B.n == 128) {
         batch_pass<8, 16, 16, true, 128>(B, level, tile);
       } else if (B.var == VAR_P2 && B.n == 256) {
@@ -797,15 +617,6 @@ int autotune(dgpe_batch *b, Cls &c) {
   return set_attrs(b, c);
 }
 
-int batch_rows_bytes(int n) {
-  int b = 0;
-  with_row_length(n, [&](auto Nc) {
-    b = batch_rows_smem<decltype(Nc)::value>();
-    return cudaSuccess;
-  });
-  return b;
-}
-
 // The persistent step's data: one BProb per problem (its pass arguments at
 // the persistent tile shapes and tuned plans), one step's work list
 // (pass-major, largest problems first within a pass), the resident problems,
@@ -838,18 +649,14 @@ int build_persistent(dgpe_batch *b) {
       q.resident = (c.n == kRes && c.var == VAR_P2) ? 1 : 0;
       q.tiles[0] = ((e->nrows + 1) / 2 + LP - 1) / LP;
       q.tiles[1] = (e->ncol_spec + sW - 1) / sW;
-      q.kxr = e->row_kr; q.kxc = e->row_kc; q.kyr = e->cn_kr[1]; q.kyc = e->cn_kc[1];
-      q.rows = (c.imag ? q.kxr.dl : q.kxc.dl) > 0;
-      q.cols = (c.imag ? q.kyr.dl : q.kyc.dl) > 0 && cW * e->cn[1].TPL == DGPE_MAXT;
-      const int per_tile = kRowWarpsBatch * rows_per_tile(c.n);
-      q.tiles[2] = q.rows ? (e->nrows + per_tile - 1) / per_tile : q.tiles[0];
+      q.tiles[2] = q.tiles[0];
       q.tiles[3] = (c.n + cW - 1) / cW;
       q.per_step = q.tiles[0] + q.tiles[1] + q.tiles[2] + q.tiles[3];
       if (q.resident) res.push_back(i);
       const size_t xs = sizeof(Cx) * (size_t)(LP * e->x_pitchz + 2 * LP * e->x_pitch);
       const size_t ss = sizeof(Cx) * (size_t)c.n * sW;
       const size_t cs = sizeof(Cx) * (size_t)cW * e->cn[1].pitch;
-      if (!q.resident) smem = std::max({smem, xs, ss, cs, (size_t)(q.rows ? batch_rows_bytes(c.n) : 0)});
+      if (!q.resident) smem = std::max(smem, std::max(xs, std::max(ss, cs)));
     }
   }
   // one step's items, pass-major, largest problems first within a pass

@@ -959,39 +959,6 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
   if (t == 0) { mbar_inval(&bar[0]); mbar_inval(&bar[1]); }
 }
 
-// Last pass of the step, block bid of nblk: norm partials (imaginary time) and,
-// in the last block to finish, the deterministic FP64 total, the new scale and
-// the step counter.
-template <typename R>
-__device__ __forceinline__ void cn_final(const CArgs<R> &A, double acc, unsigned nblk, unsigned bid, double *red, int &am_last) {
-  if (A.norm) {
-    double s = block_sum(acc, red);
-    if (threadIdx.x == 0) A.partial[bid] = s;
-  }
-  if (threadIdx.x == 0) {
-    __threadfence();
-    const unsigned ticket = atomicAdd(A.counter, 1u);
-    am_last = (ticket == nblk - 1);
-  }
-  __syncthreads();
-  if (!am_last) return;
-  __threadfence();
-  if (A.norm) {
-    double s = 0.0;
-    for (unsigned i = threadIdx.x; i < nblk; i += blockDim.x) s += __ldcg(A.partial + i);
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) {
-      const double norm = A.prm[PRM_CELL] * s;
-      if (norm > 0.0 && isfinite(norm)) A.prm[PRM_SC] = 1.0 / sqrt(norm);
-      else A.prm[PRM_NONFINITE] = 1.0;
-    }
-  }
-  if (threadIdx.x == 0) {
-    *A.step += 1;
-    *A.counter = 0u;
-  }
-}
-
 // ------------------------------------------------------- P2 / P3 (strided)
 // NORM false: a pass without the norm (no |x|^2 code at all); true: the
 // runtime flag A.norm decides.
@@ -1053,7 +1020,37 @@ __device__ __forceinline__ void cn_strided_body(const CArgs<R> &A, int bx, int b
     acc = (double)ts;
   }
   if (!A.final_pass) return;
-  cn_final(A, acc, (unsigned)(gx * gy), (unsigned)(by * gx + bx), red, am_last);
+  // Last pass of the step: norm partials (imaginary time) and, in the last
+  // block to finish, the deterministic FP64 total, the new scale and the
+  // step counter.
+  const unsigned nblk = (unsigned)(gx * gy);
+  const unsigned bid = (unsigned)(by * gx + bx);
+  if (A.norm) {
+    double s = block_sum(acc, red);
+    if (threadIdx.x == 0) A.partial[bid] = s;
+  }
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned ticket = atomicAdd(A.counter, 1u);
+    am_last = (ticket == nblk - 1);
+  }
+  __syncthreads();
+  if (!am_last) return;
+  __threadfence();
+  if (A.norm) {
+    double s = 0.0;
+    for (unsigned i = threadIdx.x; i < nblk; i += blockDim.x) s += __ldcg(A.partial + i);
+    s = block_sum(s, red);
+    if (threadIdx.x == 0) {
+      const double norm = A.prm[PRM_CELL] * s;
+      if (norm > 0.0 && isfinite(norm)) A.prm[PRM_SC] = 1.0 / sqrt(norm);
+      else A.prm[PRM_NONFINITE] = 1.0;
+    }
+  }
+  if (threadIdx.x == 0) {
+    *A.step += 1;
+    *A.counter = 0u;
+  }
 }
 template <typename R, typename Coef, int CL, bool NORM = true>
 __global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB(R)) k_cn_strided_batch(const CArgs<R> *__restrict__ args) {
