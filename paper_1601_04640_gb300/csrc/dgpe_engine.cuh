@@ -548,7 +548,12 @@ template <typename R> struct EngineT : Engine {
 
   // The FP64 form solves each line serially once there are enough lines for
   // one warp per SM sub-partition at least (it is FP64-pipe-bound, and the
-  // serial solve does half the arithmetic); flags force either form.
+  // serial solve does half the arithmetic); flags force either form.  The
+  // small-grid passes keep their solves, except in real time without dipoles,
+  // where a step is solves and little else (us per step, line-serial and
+  // small-grid: 96^3 250 and 268, 160 x 128 x 128 478 and 658, 160^3 711 and
+  // 1016; in imaginary time 160^3 742 and 647, with dipoles in real time 2123
+  // and 1785).
   int choose_cn_form() {
     const size_t lines_min = nsites / (size_t)std::max(nx, std::max(ny, nz));
     if ((p.flags & DGPE_FLAG_CN_SERIAL) && (p.flags & DGPE_FLAG_CN_CHUNKED)) {
@@ -563,7 +568,7 @@ template <typename R> struct EngineT : Engine {
       cn_serial = false;
     } else if (p.flags & DGPE_FLAG_CN_SERIAL) cn_serial = true;
     else if (p.flags & DGPE_FLAG_CN_CHUNKED) cn_serial = false;
-    else cn_serial = lines_min >= 8192 && !fine;
+    else cn_serial = lines_min >= 8192 && (!fine || (!imag && !has_dip));
     const int ns[3] = {nx, ny, nz};
     for (int a = 0; a < dim; ++a) {
       LnCfg &L = ln[a];
@@ -1738,7 +1743,7 @@ template <typename R> struct EngineT : Engine {
     if (rc) return rc;
     p.mode = mode;
     imag = (mode == DGPE_IMAG);
-    if ((rc = build_cn_tables())) return rc;
+    if ((rc = choose_cn_form()) || (rc = build_cn_tables())) return rc;
     setup_lines();
     if (use_graph && (rc = capture())) return rc;
     return DGPE_OK;
