@@ -10,13 +10,15 @@ namespace {
 
 // Columns per block of 256 threads: 8 (32 chunks) to 128 (2 chunks), halved
 // while a grid leaves SMs without a block, to blocks of one warp or segments of
-// two columns.
+// two columns; the table form to 128 threads, because every block brings in the
+// whole of the tables (512 x 512 in real time: two columns per block 14.3 us,
+// four 10.2).
 constexpr int kColsThreads = 256;
-inline int cols_lw(int n, int cl, unsigned tot, int nsm) {
-  const int tpl = n / cl;
+inline int cols_lw(int n, int cl, unsigned tot, int nsm, bool tab) {
+  const int tpl = n / cl, least = tab ? 128 : 32;
   int lw = 0;
   while ((2 << lw) * tpl <= kColsThreads) ++lw;
-  while (lw > 1 && (1 << lw) * tpl > 32 && (tot >> lw) < (unsigned)nsm) --lw;
+  while (lw > 1 && (1 << lw) * tpl > least && (tot >> lw) < (unsigned)nsm) --lw;
   return lw;
 }
 
@@ -168,7 +170,7 @@ template <typename Coef, class F> cudaError_t with_kernel(int cl, bool norm, boo
   });
 }
 template <typename Coef> int grid_of(int n, int cl, unsigned tot, int nsm, bool tab) {
-  const int w = 1 << cols_lw(n, cl, tot, nsm), T = w * (n / cl), ntiles = (int)((tot + (unsigned)w - 1) / (unsigned)w);
+  const int w = 1 << cols_lw(n, cl, tot, nsm, tab), T = w * (n / cl), ntiles = (int)((tot + (unsigned)w - 1) / (unsigned)w);
   int occ = 0;
   with_kernel<Coef>(cl, true, tab, [&](auto k) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, T, cols_smem<Coef>(n, T, tab));
@@ -176,9 +178,9 @@ template <typename Coef> int grid_of(int n, int cl, unsigned tot, int nsm, bool 
   return std::max(1, std::min(ntiles, nsm * std::max(occ, 1)));
 }
 template <typename Coef> cudaError_t launch(const ColArgs &A, const CnConst<Coef> &K, int grid, cudaStream_t s) {
-  const int lw = cols_lw(A.n, A.cl, A.tot, A.nsm), w = 1 << lw, T = w * (A.n / A.cl);
-  const int ntiles = (int)((A.tot + (unsigned)w - 1) / (unsigned)w);
   const bool tab = K.dl == 0;
+  const int lw = cols_lw(A.n, A.cl, A.tot, A.nsm, tab), w = 1 << lw, T = w * (A.n / A.cl);
+  const int ntiles = (int)((A.tot + (unsigned)w - 1) / (unsigned)w);
   return with_kernel<Coef>(A.cl, A.norm != 0, tab, [&](auto k) {
     return launch_pdl(A.early != 0, k, dim3(grid), T, cols_smem<Coef>(A.n, T, tab), s, A, K, lw, ntiles);
   });
