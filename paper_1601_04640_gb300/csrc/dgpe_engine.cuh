@@ -218,13 +218,14 @@ constexpr size_t kRunSites = (size_t)1 << 22;
 // time, the other passes first): 64 x 64 x 48 191 -> 109, 64 x 80 x 64 250 ->
 // 172, 96^3 465 -> 420, but 128 x 96 x 96 512 -> 540: up to 2^20 sites.  Where
 // every length is a power of two up to 128 the other passes' FMA-form
-// transforms win from 2^18 (64^3 184 -> 196, 128 x 128 x 64 463 -> 472); where
-// nx is 5 2^k their 20 points per thread spill and they lose to the end of the
-// range (160^3 2239 -> 1950).
+// transforms win from 2^20 (64^3 183 -> 158, 128 x 64 x 64 281 -> 259, but 64 x
+// 128 x 128 462 -> 495; in imaginary time 144 -> 127, 210 -> 202, 463 -> 432);
+// where nx is 5 2^k their 20 points per thread spill and they lose to the end
+// of the range (160^3 2239 -> 1950).
 inline size_t fine_sites(int nx, int ny, int nz) {
   auto small2 = [](int n) { return is_pow2(n) && n <= 128; };
   if (nx % 5 == 0) return (size_t)1 << 23;
-  return small2(nx) && small2(ny) && small2(nz) && nz > 1 ? ((size_t)1 << 18) - 1 : (size_t)1 << 20;
+  return small2(nx) && small2(ny) && small2(nz) && nz > 1 ? (size_t)1 << 19 : (size_t)1 << 20;
 }
 // Call f(N, EPT) for any line length of the FP32 strided transforms (EPT
 // elements per thread: 16, 12 or 20 for 2^k, 3 2^k, 5 2^k).

@@ -41,3 +41,28 @@ def test_real_time_without_dipoles_solves_lines_serially(n, serial):
         e = np.linalg.norm(s.get_psi() - ref) / np.linalg.norm(ref)
         print(n, "rel L2", e)
         assert e < 15 * 100 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("form", ["imag", "imag real state", "real"])
+@pytest.mark.parametrize("n", [(64, 64, 64), (128, 32, 64), (32, 128, 128), (128, 64, 64), (64, 128, 128)])
+def test_power_of_two_boxes_on_both_sides_of_the_small_grid_passes(n, form):
+    """2^18 and 2^19 sites take the small-grid passes, 2^20 the others; exponents on both sides of 1/8."""
+    dgpe = _dgpe()
+    from paper_1601_04640_gb300 import synth
+    imag, real_psi = form != "real", form == "imag real state"
+    h, nu, g, gdd, dt = (0.2, 0.25, 0.22), (1.0, 1.3, 0.8), 40.0, 8.0, 2e-3
+    psi0 = synth.gaussian_state(n, h, nu, 0.0 if real_psi else 0.01, 3)
+    if real_psi:
+        psi0 = psi0.real.astype(complex)
+    op = oracle.Params(dim=3, n=n, h=h, nu=nu, g=g, gdd=gdd, dt=dt, imag=imag, kernel="dipolar3d")
+    with dgpe.Solver(3, n, h, nu, g, gdd, dt, imag, True, real_psi=real_psi) as s:
+        s.set_psi(psi0)
+        s.step(5)  # one run of several steps and a single one
+        psi, o = s.get_psi(), s.observables()
+    ref = oracle.step(op, psi0, 0, 5)
+    r = oracle.observables(op, ref, 5)
+    e = np.linalg.norm(psi - ref) / np.linalg.norm(ref)
+    print(n, form, "rel L2", e, "energy", o["energy"] / r["energy"] - 1)
+    assert e < 5 * 100 * 2.0 ** -53
+    for k in ("norm", "energy", "mu", "kin", "pot", "contact", "rms_r"):
+        assert abs(o[k] - r[k]) <= 1e-11 * abs(r[k])
