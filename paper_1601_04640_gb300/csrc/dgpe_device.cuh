@@ -84,8 +84,9 @@ static __device__ __noinline__ float expm1_call(float a) { return expm1f(a); }
 // a^10 / 10! in FP64 and a^6 / 6! in FP32 (first omitted terms 2.3e-17 and
 // 7.6e-10 relative at 1/8), which is 10 and 6 multiply-adds; beyond that the
 // library function.  A step's exponents are dt (V + ...), mostly far below 1/8.
+// FP64 tests the high word: a compare would be one of some 13 FP64 operations.
 __device__ __forceinline__ double fexpm1(double a) {
-  if (!(fabs(a) <= 0.125)) return expm1_call(a);
+  if ((__double2hiint(a) & 0x7fffffff) >= 0x3fc00000) return expm1_call(a);  // |a| >= 1/8, NaN
   double p = 1.0 / 3628800.0;
   p = fma(p, a, 1.0 / 362880.0);
   p = fma(p, a, 1.0 / 40320.0);
