@@ -201,14 +201,15 @@ template <class F> int with_pow2_len(int n, F &&f) {
 // Largest grid whose passes start while the one before drains: the pass ahead
 // has to leave the SMs room, or blocks that arrive early take it from that
 // pass's own.  us per step in imaginary / real time, in order first:
-//   FP64 with dipoles   32^3 49.6 / 55.0 -> 46.5 / 53.9, but 48^3 70.8 / 80.9 ->
-//     75.1 / 100, 128 x 40 x 48 103 / 128 -> 128 / 181, 64^3 142 / 187 -> 151 / 198;
+//   FP64 with dipoles   32^3 49.6 / 55.0 -> 46.5 / 53.9, 40^3 - / 64.8 -> - / 61.3,
+//     but 48^3 70.8 / 80.9 -> 75.1 / 100, 128 x 40 x 48 103 / 128 -> 128 / 181,
+//     384 x 512 85.8 / 102 -> 148 / 169;
 //   FP64 without        48^3 36.7 / 46.8 -> 35.5 / 45.7, 64 x 64 x 32 39.1 / 49.3 ->
 //     37.6 / 48.0, but 384 x 512 46.7 / 62.7 -> 52.4 / 71.9;
 //   FP32                64^3 29.4 / 28.7 -> 28.1 / 27.3, but 128^3 51 -> 59 and,
 //     without dipoles, 320 x 512 14.5 / 13.0 -> 15.9 / 14.0.
 inline size_t early_sites(bool fp64, int dim, bool dip) {
-  if (fp64) return dip ? (size_t)1 << 15 : (size_t)1 << 17;
+  if (fp64) return dip ? (size_t)1 << 16 : (size_t)1 << 17;
   return dim == 2 && !dip ? ((size_t)1 << 17) - 1 : (size_t)1 << 18;
 }
 // largest grid with a graph of several steps: above it a step takes some 100 us,
