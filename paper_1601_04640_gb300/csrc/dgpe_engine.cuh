@@ -293,18 +293,17 @@ template <typename R> struct EngineT : Engine {
   // pass configurations
   int x_LP = 0, x_T = 0, x_TPL = 0, x_C = 0, x_pitchz = 0, x_pitch = 0, x_grid = 0;
   size_t x_smem = 0, x4_smem = 0;  // the C2R/exp/CN pass; the density pass (Z tile only)
-  // FP32 bulk, complex state, power-of-two nx: the pipelined x-line pass
-  // (k_p1_pipe, persistent CTAs fed by bulk copies); grid and shared memory
+  // FP32 bulk, complex state, power-of-two nx, slowly decaying coefficients:
+  // the pipelined x-line pass (k_p1_pipe, persistent CTAs fed by bulk copies);
+  // grid and shared memory
   bool p1_pipe = false;
   int p1_grid[2] = {0, 0};  // real, complex CN coefficients
   size_t p1_smem[2] = {0, 0};
   // FP32 bulk: the warp-per-tile x-row passes (dgpe_rows*.cu); persistent
   // grids by forward source and backward mode (ROWS_STEP: imaginary time
-  // first, real time last), constant CN forms along x, tensor map of psi
+  // first, real time last), tensor map of psi
   bool rows_fwd = false, rows_back = false;
   int rows_fgrid[3] = {0, 0, 0}, rows_bgrid[ROWS_MODES + 1] = {0};
-  CnConst<float> row_kr{};
-  CnConst<float2> row_kc{}, row_ka{};
   CUtensorMap tm_psi{};
   // ... and the TMA-tiled strided transforms (k_fft_tma): tensor maps of the
   // half spectrum for lines along y and along z
@@ -820,15 +819,12 @@ template <typename R> struct EngineT : Engine {
         if (dl >= 64) dl = 0;
       }
       cn_dlim[a] = dl;
-      if (a == 0 && sizeof(R) == 4) {
-        const int cl = rows_chunk(n);
-        row_kr = cn_const<float>(zd(tau[0], 0.0), cl, n / cl);
-        row_kc = cn_const<float2>(zd(0.0, tau[0]), cl, n / cl);
-        row_ka = cn_const<float2>(zd(0.0, -tau[0]), cl, n / cl);
+      if constexpr (sizeof(R) == 4) {
+        const int cl = a == 0 ? rows_chunk(n) : C;
+        cn_kr[a] = cn_const<float>(zd(tau[a], 0.0), cl, n / cl);
+        cn_kc[a] = cn_const<float2>(zd(0.0, tau[a]), cl, n / cl);
+        cn_ka[a] = cn_const<float2>(zd(0.0, -tau[a]), cl, n / cl);
       }
-      cn_kr[a] = cn_const<float>(zd(tau[a], 0.0), C, n / C);
-      cn_kc[a] = cn_const<float2>(zd(0.0, tau[a]), C, n / C);
-      cn_ka[a] = cn_const<float2>(zd(0.0, -tau[a]), C, n / C);
       if (!cntab[a]) {
         int rc = dalloc((Cx **)&cntab[a], 4 * (size_t)n + 1);
         if (rc) return rc;
@@ -935,36 +931,37 @@ template <typename R> struct EngineT : Engine {
       rc = with_svar<EPT_S>(var[a], [&](auto EPc, auto P2c) -> int {
         constexpr int EP = decltype(EPc)::value;
         constexpr bool P2 = decltype(P2c)::value;
-      constexpr bool FM = P2 && (sizeof(R) == 8 || DGPE_FFT_FMA_F32);  // FMA-form twiddled stages
-      constexpr bool FM1 = P2 && sizeof(R) == 8;  // the C2R pass: FP64 only
+        constexpr bool FM = P2 && (sizeof(R) == 8 || DGPE_FFT_FMA_F32);  // FMA-form twiddled stages
         int r;
-        if ((r = smem_attr(k_fft_strided<R, EP, 0, P2, FM>, fs))) return r;
-        if ((r = smem_attr(k_fft_strided<R, EP, 1, P2, FM>, fs))) return r;
-        if ((r = smem_attr(k_fft_strided<R, EP, 2, P2, FM>, fs))) return r;
+        if constexpr (sizeof(R) == 8) {
+          if ((r = smem_attr(k_fft_strided<R, EP, 0, P2, FM>, fs))) return r;
+          if ((r = smem_attr(k_fft_strided<R, EP, 1, P2, FM>, fs))) return r;
+          if ((r = smem_attr(k_fft_strided<R, EP, 2, P2, FM>, fs))) return r;
+        }
         if ((r = smem_attr(k_fft_strided<R, EP, 3, P2, FM>, fs))) return r;
         return DGPE_OK;
       });
       if (rc) return rc;
-      if constexpr (sizeof(R) == 4) continue;  // FP32: dgpe_cols.cu
-      rc = with_cl(var[a], [&](auto CLc) -> int {
-        constexpr int CL = decltype(CLc)::value;
-        int r;
-        const size_t two = 2 * cn[a].smem;
-        if ((r = smem_attr(k_cn_strided_pipe<R, R, CL>, two))) return r;
-        if ((r = smem_attr(k_cn_strided_pipe<R, Cx, CL>, two))) return r;
-        if ((r = smem_attr(k_cn_strided_pipe<R, R, CL, false>, two))) return r;
-        if ((r = smem_attr(k_cn_strided_pipe<R, Cx, CL, false>, two))) return r;
-        // persistent grid: as many CTAs as fit on the device, at most one per
-        // tile, each double-buffered (the next tile is prefetched)
-        const int ntiles = (int)(cn[a].grid.x * cn[a].grid.y);
-        int occ = 0;
-        DGPE_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cn_strided_pipe<R, R, CL>, cn[a].T, two));
-        cn[a].pgrid[0] = std::max(1, std::min(ntiles, nsm * std::max(occ, 1)));
-        DGPE_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cn_strided_pipe<R, Cx, CL, false>, cn[a].T, two));
-        cn[a].pgrid[1] = std::max(1, std::min(ntiles, nsm * std::max(occ, 1)));
-        return DGPE_OK;
-      });
-      if (rc) return rc;
+      if constexpr (sizeof(R) == 8) {  // FP32: dgpe_cols.cu
+        rc = with_cl(var[a], [&](auto CLc) -> int {
+          constexpr int CL = decltype(CLc)::value;
+          int r;
+          const size_t two = 2 * cn[a].smem;
+          if ((r = smem_attr(k_cn_strided_pipe<double, CL, true>, two))) return r;
+          if ((r = smem_attr(k_cn_strided_pipe<double, CL, false>, two))) return r;
+          if ((r = smem_attr(k_cn_strided_pipe<double2, CL, false>, two))) return r;
+          // persistent grid: as many CTAs as fit on the device, at most one per
+          // tile, each double-buffered (the next tile is prefetched)
+          const int ntiles = (int)(cn[a].grid.x * cn[a].grid.y);
+          int occ = 0;
+          DGPE_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cn_strided_pipe<double, CL, true>, cn[a].T, two));
+          cn[a].pgrid[0] = std::max(1, std::min(ntiles, nsm * std::max(occ, 1)));
+          DGPE_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cn_strided_pipe<double2, CL, false>, cn[a].T, two));
+          cn[a].pgrid[1] = std::max(1, std::min(ntiles, nsm * std::max(occ, 1)));
+          return DGPE_OK;
+        });
+        if (rc) return rc;
+      }
     }
     if ((rc = setup_rows())) return rc;
     return setup_tma();
@@ -1033,36 +1030,28 @@ template <typename R> struct EngineT : Engine {
     A.uny = ny;
     return A;
   }
-  // FP32, modes 0-2: the length-specialised transform fed by registers
+  // FP32, modes 0-2: the length-specialised transform fed by registers.  A
+  // plane's one strided pass has few tiles (9 of 16 columns at 256^2): tiles
+  // of one warp, or of two columns, spread over more SMs (the one-shot flag
+  // keeps the wide ones).
+  static constexpr int narrow_width(int n, int ept) { return 32 * ept / n > 2 ? 32 * ept / n : 2; }
   bool launch_fft_ct(const FtCfg &f, int mode, const SArgs<R> &A, cudaStream_t s) {
     if constexpr (sizeof(R) != 4) {
       return false;
     } else {
       if (mode > 2) return false;
-      bool done = false;
       with_col_len(f.n, [&](auto Nc, auto Ec) -> int {
         constexpr int N = decltype(Nc)::value, E = decltype(Ec)::value, WW = col_width(N, E), WN = narrow_width(N, E);
-        if (f.W != WW) return 0;
-        if (narrow(f, mode)) {
+        if (dim == 2 && !(p.flags & DGPE_FLAG_P1_ONESHOT))
           launch_pdl(early, k_fft_strided_ct<E, 2, N, WN>, dim3((ncol_spec + WN - 1) / WN), WN * N / E,
                      sizeof(Cx) * (size_t)WN * N, s, A);
-          done = true;
-          return 0;
-        }
-        if (mode == 0) launch_pdl(early, k_fft_strided_ct<E, 0, N, WW>, f.grid, f.T, f.smem, s, A);
+        else if (mode == 0) launch_pdl(early, k_fft_strided_ct<E, 0, N, WW>, f.grid, f.T, f.smem, s, A);
         else if (mode == 1) launch_pdl(early, k_fft_strided_ct<E, 1, N, WW>, f.grid, f.T, f.smem, s, A);
         else launch_pdl(early, k_fft_strided_ct<E, 2, N, WW>, f.grid, f.T, f.smem, s, A);
-        done = true;
         return 0;
       });
-      return done;
+      return true;
     }
-  }
-  // A plane's one strided pass has few tiles (9 of 16 columns at 256^2): tiles
-  // of one warp, or of two columns, where they spread over more SMs.
-  static constexpr int narrow_width(int n, int ept) { return 32 * ept / n > 2 ? 32 * ept / n : 2; }
-  bool narrow(const FtCfg &f, int mode) const {
-    return !(p.flags & DGPE_FLAG_P1_ONESHOT) && dim == 2 && mode == 2 && (int)f.grid.x < nsm;
   }
   // Tile width of a strided FP32 transform: DGPE_W_FFT_F32 columns, halved
   // until a block has at most DGPE_MAXT_FFT threads.
@@ -1071,21 +1060,20 @@ template <typename R> struct EngineT : Engine {
     while (w > 1 && w * n / ept > DGPE_MAXT_FFT) w >>= 1;
     return w;
   }
-  // FP32: tensor maps of the half spectrum (kx, y, z; kx valid columns, rows
-  // of px elements) for the TMA-tiled transforms.  Not fatal when
-  // unavailable: the length-specialised kernels run instead.
+  // FP32 boxes: tensor maps of the half spectrum (kx, y, z; kx valid columns,
+  // rows of px elements) for the TMA-tiled transforms: FFT_y and IFFT_y along
+  // y, FFT_z.U.IFFT_z along z.  Not fatal when unavailable: the
+  // length-specialised kernels run instead.
   int tma_grid[2] = {0, 0};
   template <int AX, int N, int E> int tma_attrs(int &grid) {
-    constexpr int WW = col_width(N, E);
+    constexpr int WW = col_width(N, E), FIRST = AX == 1 ? 0 : 2;
     const size_t sm = 2 * sizeof(Cx) * (size_t)WW * N + 128;
     int r;
-    if constexpr (AX == 1) {  // lines along y: FFT_y, IFFT_y (3D) and FFT_y.U.IFFT_y (2D)
-      if ((r = smem_attr(k_fft_tma<E, 0, N, WW, AX>, sm))) return r;
+    if ((r = smem_attr(k_fft_tma<E, FIRST, N, WW, AX>, sm))) return r;
+    if constexpr (AX == 1)
       if ((r = smem_attr(k_fft_tma<E, 1, N, WW, AX>, sm))) return r;
-    }
-    if ((r = smem_attr(k_fft_tma<E, 2, N, WW, AX>, sm))) return r;
     int occ = 0;
-    DGPE_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_fft_tma<E, 2, N, WW, AX>, WW * N / E, sm));
+    DGPE_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_fft_tma<E, FIRST, N, WW, AX>, WW * N / E, sm));
     grid = nsm * occ;
     return DGPE_OK;
   }
@@ -1099,32 +1087,24 @@ template <typename R> struct EngineT : Engine {
       return DGPE_OK;
     } else {
       tma_fft = false;
-      if (!has_dip || (p.flags & DGPE_FLAG_P1_ONESHOT)) return DGPE_OK;
+      if (!has_dip || dim == 2 || (p.flags & DGPE_FLAG_P1_ONESHOT)) return DGPE_OK;
       TensorMapEncodeTiledFn enc = tensor_map_encoder();
       if (!enc) return DGPE_OK;
       const cuuint64_t dims[3] = {(cuuint64_t)ncol_spec, (cuuint64_t)ny, (cuuint64_t)nz};
       const cuuint64_t strides[2] = {(cuuint64_t)px * sizeof(Cx), (cuuint64_t)ny * px * sizeof(Cx)};
       const cuuint32_t es[3] = {1, 1, 1};
       auto rows = [](int n) { return (cuuint32_t)(n / ((n + 255) / 256)); };
-      const cuuint32_t by[3] = {(cuuint32_t)fy.W, rows(ny), 1};
-      if (enc(&tm_y, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, spec, dims, strides, by, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return DGPE_OK;
-      if (dim == 3) {
-        const cuuint32_t bz[3] = {(cuuint32_t)fz.W, 1, rows(nz)};
-        if (enc(&tm_z, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, spec, dims, strides, bz, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-          return DGPE_OK;
-      }
+      const cuuint32_t by[3] = {(cuuint32_t)fy.W, rows(ny), 1}, bz[3] = {(cuuint32_t)fz.W, 1, rows(nz)};
+      auto encode = [&](CUtensorMap *tm, const cuuint32_t *box) {
+        return enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, spec, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+      };
+      if (!encode(&tm_y, by) || !encode(&tm_z, bz)) return DGPE_OK;
       int r = this->template tma_axis<1>(fy, tma_grid[0]);
+      if (!r) r = this->template tma_axis<2>(fz, tma_grid[1]);
       if (r) return r;
-      if (dim == 3) {
-        r = this->template tma_axis<2>(fz, tma_grid[1]);
-          if (r) return r;
-      }
-      tma_fft = tma_grid[0] > 0 && (dim == 2 || tma_grid[1] > 0);
+      tma_fft = tma_grid[0] > 0 && tma_grid[1] > 0;
       return DGPE_OK;
     }
   }
@@ -1132,17 +1112,16 @@ template <typename R> struct EngineT : Engine {
     if constexpr (sizeof(R) != 4) {
       return false;
     } else {
-      if (!tma_fft || mode > 2 || (f.axis == 2 && mode != 2) || narrow(f, mode)) return false;
+      if (!tma_fft || mode > 2 || (f.axis == 2) != (mode == 2)) return false;
       const int ncb = (int)f.grid.x, ntiles = (int)(f.grid.x * f.grid.y);
       const int g = std::max(1, std::min(ntiles, tma_grid[f.axis - 1]));
       double *tf = prm + PRM_TIMEOUT;
       with_col_len(f.n, [&](auto Nc, auto Ec) -> int {
         constexpr int N = decltype(Nc)::value, E = decltype(Ec)::value, WW = col_width(N, E), T = WW * N / E;
         const size_t sm = 2 * sizeof(Cx) * (size_t)WW * N + 128;
-        if (f.axis == 2) launch_pdl(early, k_fft_tma<E, 2, N, WW, 2>, dim3(g), T, sm, s, tm_z, A, ncb, ntiles, tf);
+        if (mode == 2) launch_pdl(early, k_fft_tma<E, 2, N, WW, 2>, dim3(g), T, sm, s, tm_z, A, ncb, ntiles, tf);
         else if (mode == 0) launch_pdl(early, k_fft_tma<E, 0, N, WW, 1>, dim3(g), T, sm, s, tm_y, A, ncb, ntiles, tf);
-        else if (mode == 1) launch_pdl(early, k_fft_tma<E, 1, N, WW, 1>, dim3(g), T, sm, s, tm_y, A, ncb, ntiles, tf);
-        else launch_pdl(early, k_fft_tma<E, 2, N, WW, 1>, dim3(g), T, sm, s, tm_y, A, ncb, ntiles, tf);
+        else launch_pdl(early, k_fft_tma<E, 1, N, WW, 1>, dim3(g), T, sm, s, tm_y, A, ncb, ntiles, tf);
         return 0;
       });
       return true;
@@ -1165,13 +1144,12 @@ template <typename R> struct EngineT : Engine {
       constexpr int EP = decltype(EPc)::value;
       constexpr bool P2 = decltype(P2c)::value;
       constexpr bool FM = P2 && (sizeof(R) == 8 || DGPE_FFT_FMA_F32);  // FMA-form twiddled stages
-      constexpr bool FM1 = P2 && sizeof(R) == 8;  // the C2R pass: FP64 only
-      switch (mode) {
-        case 0: launch_pdl(early, k_fft_strided<R, EP, 0, P2, FM>, f.grid, f.T, f.smem, s, A); break;
-        case 1: launch_pdl(early, k_fft_strided<R, EP, 1, P2, FM>, f.grid, f.T, f.smem, s, A); break;
-        case 2: launch_pdl(early, k_fft_strided<R, EP, 2, P2, FM>, f.grid, f.T, f.smem, s, A); break;
-        default: launch_pdl(early, k_fft_strided<R, EP, 3, P2, FM>, f.grid, f.T, f.smem, s, A); break;
+      if constexpr (sizeof(R) == 8) {
+        if (mode == 0) launch_pdl(early, k_fft_strided<R, EP, 0, P2, FM>, f.grid, f.T, f.smem, s, A);
+        if (mode == 1) launch_pdl(early, k_fft_strided<R, EP, 1, P2, FM>, f.grid, f.T, f.smem, s, A);
+        if (mode == 2) launch_pdl(early, k_fft_strided<R, EP, 2, P2, FM>, f.grid, f.T, f.smem, s, A);
       }
+      if (mode == 3) launch_pdl(early, k_fft_strided<R, EP, 3, P2, FM>, f.grid, f.T, f.smem, s, A);
       return DGPE_OK;
     });
     launched(1);
@@ -1233,15 +1211,15 @@ template <typename R> struct EngineT : Engine {
       A.dtf = dtf;
       if (phi_out) A.phi_out = phi_out;
       if (A.mode == ROWS_PHI) {
-        e = rows_back_launch(A, tm_psi, row_kr, rows_bgrid[ROWS_PHI], s);
+        e = rows_back_launch(A, tm_psi, cn_kr[0], rows_bgrid[ROWS_PHI], s);
         return true;
       }
       if (imag) {
-        if (mode != 0 || row_kr.dl == 0) return false;
-        e = rows_back_launch(A, tm_psi, row_kr, rows_bgrid[A.mode], s);
+        if (mode != 0 || cn_kr[0].dl == 0) return false;
+        e = rows_back_launch(A, tm_psi, cn_kr[0], rows_bgrid[A.mode], s);
         return true;
       }
-      const CnConst<float2> &K = mode == 2 ? row_ka : row_kc;
+      const CnConst<float2> &K = mode == 2 ? cn_ka[0] : cn_kc[0];
       if (K.dl == 0 && mode != 3) return false;
       CUtensorMap tm = tm_psi;
       if (buf && buf != psi) {
@@ -1255,33 +1233,36 @@ template <typename R> struct EngineT : Engine {
   }
   int launch_cn(int axis, bool final_pass, cudaStream_t s, Cx *buf = nullptr, bool adjoint = false) {
     if (cn_serial) return launch_lines(axis, final_pass, s, buf, adjoint);
-    if constexpr (sizeof(R) == 4) return launch_cols(axis, final_pass, s, buf, adjoint);
-    cudaError_t e = cudaSuccess;
-    if (fine_solve(axis, final_pass, s, buf, adjoint, e)) {
+    if constexpr (sizeof(R) == 4) {
+      return launch_cols(axis, final_pass, s, buf, adjoint);
+    } else {
+      cudaError_t e = cudaSuccess;
+      if (fine_solve(axis, final_pass, s, buf, adjoint, e)) {
+        launched(1);
+        DGPE_CK(e);
+        return DGPE_OK;
+      }
+      const CnCfg &c = cn[axis];
+      CArgs<R> A{};
+      A.psi = buf ? buf : psi; A.cntab = adjoint ? cntab_adj[axis] : cntab[axis];
+      A.prm = prm; A.partial = partial; A.counter = counter;
+      A.step = dstep; A.estride = c.es; A.ostride = c.os; A.n = c.n; A.ncols = c.ncols; A.W = c.W;
+      A.TPL = c.TPL; A.C = c.C; A.pitch = c.pitch; A.final_pass = final_pass ? 1 : 0;
+      A.norm = (final_pass && imag) ? 1 : 0; A.tau = adjoint ? -tau[axis] : tau[axis];
+      A.cnd = cn_dlim[axis];
+      const int ncb = (int)c.grid.x, ntiles = (int)(c.grid.x * c.grid.y);
+      with_cl(var[axis], [&](auto CLc) -> int {
+        constexpr int CL = decltype(CLc)::value;
+        // the norm's code only in the pass that takes the norm
+        if (imag && A.norm) launch_pdl(early, k_cn_strided_pipe<double, CL, true>, dim3(c.pgrid[0]), c.T, 2 * c.smem, s, A, ncb, ntiles);
+        else if (imag) launch_pdl(early, k_cn_strided_pipe<double, CL, false>, dim3(c.pgrid[0]), c.T, 2 * c.smem, s, A, ncb, ntiles);
+        else launch_pdl(early, k_cn_strided_pipe<double2, CL, false>, dim3(c.pgrid[1]), c.T, 2 * c.smem, s, A, ncb, ntiles);
+        return DGPE_OK;
+      });
       launched(1);
-      DGPE_CK(e);
+      DGPE_LCK(__func__);
       return DGPE_OK;
     }
-    const CnCfg &c = cn[axis];
-    CArgs<R> A{};
-    A.psi = buf ? buf : psi; A.cntab = adjoint ? cntab_adj[axis] : cntab[axis];
-    A.prm = prm; A.partial = partial; A.counter = counter;
-    A.step = dstep; A.estride = c.es; A.ostride = c.os; A.n = c.n; A.ncols = c.ncols; A.W = c.W;
-    A.TPL = c.TPL; A.C = c.C; A.pitch = c.pitch; A.final_pass = final_pass ? 1 : 0;
-    A.norm = (final_pass && imag) ? 1 : 0; A.tau = adjoint ? -tau[axis] : tau[axis];
-    A.cnd = cn_dlim[axis];
-    const int ncb = (int)c.grid.x, ntiles = (int)(c.grid.x * c.grid.y);
-    with_cl(var[axis], [&](auto CLc) -> int {
-      constexpr int CL = decltype(CLc)::value;
-      // the norm's code only in the pass that takes the norm
-      if (imag && A.norm) launch_pdl(early, k_cn_strided_pipe<R, R, CL, true>, dim3(c.pgrid[0]), c.T, 2 * c.smem, s, A, ncb, ntiles);
-      else if (imag) launch_pdl(early, k_cn_strided_pipe<R, R, CL, false>, dim3(c.pgrid[0]), c.T, 2 * c.smem, s, A, ncb, ntiles);
-      else launch_pdl(early, k_cn_strided_pipe<R, Cx, CL, false>, dim3(c.pgrid[1]), c.T, 2 * c.smem, s, A, ncb, ntiles);
-      return DGPE_OK;
-    });
-    launched(1);
-    DGPE_LCK(__func__);
-    return DGPE_OK;
   }
   int launch_lines(int axis, bool final_pass, cudaStream_t s, Cx *buf, bool adjoint) {
     const LnCfg &L = ln[axis];
@@ -1313,7 +1294,6 @@ template <typename R> struct EngineT : Engine {
       constexpr int EX = decltype(EXc)::value;
       constexpr bool P2 = decltype(P2c)::value;
       constexpr bool FM = P2 && (sizeof(R) == 8 || DGPE_FFT_FMA_F32);  // FMA-form twiddled stages
-      constexpr bool FM1 = P2 && sizeof(R) == 8;  // the C2R pass: FP64 only
       if (dens_in) launch_pdl(early, k_dens_r2c_x<R, EX, 1, P2, FM>, dim3(x_grid), x_T, x4_smem, s, A);
       else if (rpsi && !src) launch_pdl(early, k_dens_r2c_x<R, EX, 2, P2, FM>, dim3(x_grid), x_T, x4_smem, s, A);
       else launch_pdl(early, k_dens_r2c_x<R, EX, 0, P2, FM>, dim3(x_grid), x_T, x4_smem, s, A);

@@ -200,15 +200,11 @@ template <typename R> struct Pad { static constexpr int W = 128 / (int)sizeof(cx
 #ifndef DGPE_MINB_P1_F32
 #define DGPE_MINB_P1_F32 3
 #endif
-#ifndef DGPE_MINB_CN_F32
-#define DGPE_MINB_CN_F32 2
-#endif
 #define DGPE_MINB_P1(R) (sizeof(R) == 4 ? DGPE_MINB_P1_F32 : 2)
 #ifndef DGPE_MINB_P4_F64
 #define DGPE_MINB_P4_F64 2
 #endif
 #define DGPE_MINB_P4(R) (sizeof(R) == 4 ? 2 : DGPE_MINB_P4_F64)
-#define DGPE_MINB_CN(R) (sizeof(R) == 4 ? DGPE_MINB_CN_F32 : 2)
 
 // Copy the n twiddles of an axis into shared memory (all threads take part;
 // the caller's next barrier publishes them).
@@ -786,9 +782,8 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, DGPE_MINB_FFT(R, EPT)) k_fft_st
 }
 
 // FP32 strided transforms (MODE 0 forward, 1 inverse, 2 forward . U .
-// inverse) with the line length N and tile width W as compile-time constants
-// (power-of-two lengths): the same arithmetic as fft_strided_body, with every
-// index folded (tile_fft_ct_cols).  Twiddles from a shared copy.
+// inverse) with the line length N and tile width W as compile-time constants:
+// every index folds (tile_fft_ct_cols).  Twiddles from a shared copy.
 template <int EPT, int MODE, int N, int W>
 __global__ void __launch_bounds__(W * N / EPT < 128 ? 64 : DGPE_MAXT_FFT, W * N / EPT < 128 ? 8 : DGPE_MINB_FFT_F32)
     k_fft_strided_ct(const __grid_constant__ SArgs<float> A) {
@@ -827,7 +822,7 @@ __global__ void __launch_bounds__(W * N / EPT < 128 ? 64 : DGPE_MAXT_FFT, W * N 
   }
 }
 
-// FP32 strided transforms with TMA tiles (power-of-two lengths): persistent
+// FP32 strided transforms of boxes with TMA tiles: persistent
 // CTAs walk the tiles; one thread loads a tile of W spectrum columns x N
 // rows into shared memory with tensor-map copies (the dense box layout
 // [row][column] is the transform's column-tile layout), two tiles ahead in
@@ -840,7 +835,7 @@ __global__ void __launch_bounds__(W * N / EPT < 128 ? 64 : DGPE_MAXT_FFT, W * N 
 #ifndef DGPE_TMA_MINB
 #define DGPE_TMA_MINB 3  // resident blocks per SM the tensor-map transforms are compiled for
 #endif
-// The 3D z-pass (MODE 2, AXIS 2) evaluates U(k) = (4 pi / 3)(3 k_z^2 / k^2 - 1)
+// The z-pass (MODE 2, AXIS 2) evaluates U(k) = (4 pi / 3)(3 k_z^2 / k^2 - 1)
 // / N_sites in FP32 from the wavenumbers (U(0) = 0) instead of reading the
 // table: four bytes less per spectrum element and no global load inside the
 // transform pair.  The pass is bound by instructions (256^3: 63 % of the issue
@@ -860,7 +855,8 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
   Cx *const buf0 = reinterpret_cast<Cx *>(smraw + ((128 - (smem_u32(smraw) & 127)) & 127));
   __shared__ unsigned long long bar[2];
   __shared__ __align__(16) Cx s_tw[N];
-  __shared__ R s_qz2[MODE == 2 && AXIS == 2 ? N : 1];  // k_z^2 of every row
+  static_assert((MODE == 2) == (AXIS == 2), "FFT_y, IFFT_y or FFT_z.U.IFFT_z");
+  __shared__ R s_qz2[MODE == 2 ? N : 1];  // k_z^2 of every row
   const int t = threadIdx.x;
   // the inverse transform runs from the last plane to the first: the x pass
   // behind it starts with the first
@@ -882,7 +878,7 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
   }
   for (int i = t; i < N; i += T) {
     s_tw[i] = A.tw[i];
-    if constexpr (MODE == 2 && AXIS == 2) {
+    if constexpr (MODE == 2) {
       const R qz = (R)((i <= N / 2) ? i : i - N) * A.uq[2];
       s_qz2[i] = qz * qz;
     }
@@ -914,7 +910,7 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
       tile_fft_ct_cols<R, N, EPT, false, W, T, true>(sm, s_tw, sload, sstore);
     } else if constexpr (MODE == 1) {
       tile_fft_ct_cols<R, N, EPT, true, W, T, true>(sm, s_tw, sload, sstore);
-    } else if constexpr (AXIS == 2) {
+    } else {
       // tile: kx = c0 + l, ky = o, kz = row a
       const int jy = (o <= A.uny / 2) ? o : o - A.uny;
       const R qy = (R)jy * A.uq[1];
@@ -923,15 +919,6 @@ __global__ void __launch_bounds__(DGPE_MAXT_FFT, EPT == 20 ? 2 : DGPE_TMA_MINB)
         const R qx = (R)(c0 + l) * dqx, qz2 = s_qz2[a], k2 = fmaf(qx, qx, qy2) + qz2;
         // 3 k_z^2 / k^2 first: a rounded 3 pref would shift the mean of U
         const R u = (k2 > (R)0) ? fmaf(pref, (R)3 * qz2 * reciprocal(k2), -pref) : (R)0;
-        sm[a * W + l] = cscale(v, u);
-      };
-      tile_fft_ct_cols<R, N, EPT, false, W, T, true>(sm, s_tw, sload, mstore);
-      tile_fft_ct_cols<R, N, EPT, true, W, T, true>(sm, s_tw, sload, sstore);
-    } else {
-      const size_t base = (size_t)o * A.ostride + c0;
-      const long long es = A.estride;
-      auto mstore = [&](int l, int a, Cx v) {
-        const R u = (c0 + l < A.ncols) ? A.U[base + a * es + l] : (R)0;
         sm[a * W + l] = cscale(v, u);
       };
       tile_fft_ct_cols<R, N, EPT, false, W, T, true>(sm, s_tw, sload, mstore);
@@ -1059,12 +1046,14 @@ __global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB(R)) k_cn_strided_batch(co
   cn_strided_body<R, Coef, CL, NORM>(A, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
 }
 
-// Persistent, double-buffered CN pass: each CTA walks tiles
+// Persistent, double-buffered CN pass of the FP64 form: each CTA walks tiles
 // blockIdx.x, blockIdx.x + gridDim.x, ...; the copies of the next tile into
 // the other shared buffer are in flight while the current tile is solved.
 // Tile id -> (column block id % nx_blocks, outer index id / nx_blocks).
-template <typename R, typename Coef, int CL, bool NORM = true>
-__global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB_CN(R)) k_cn_strided_pipe(const __grid_constant__ CArgs<R> A, int ncb, int ntiles) {
+template <typename Coef, int CL, bool NORM>
+__global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB(double))
+    k_cn_strided_pipe(const __grid_constant__ CArgs<double> A, int ncb, int ntiles) {
+  typedef double R;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double red[32];
   __shared__ int am_last;
@@ -1086,9 +1075,6 @@ __global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB_CN(R)) k_cn_strided_pipe(
     }
     cp_async_commit();
   };
-  constexpr bool TAB = (sizeof(R) == 8);
-  __shared__ __align__(16) Coef s_tab[TAB ? 1 : 4 * (512 + 512 / CL + 1)];
-  if (!TAB) stage_cn_tables<Coef, CL>(s_tab, reinterpret_cast<const Coef *>(A.cntab), n);  // visible after the loop's first barrier
   pdl_wait();
   double acc = 0.0;
   int k = 0;
@@ -1103,17 +1089,12 @@ __global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB_CN(R)) k_cn_strided_pipe(
     const int c0 = cb * W;
     cx<R> *tb = buf[k];
     const int l = threadIdx.x / A.TPL, q = threadIdx.x - l * A.TPL;
-    if constexpr (TAB) cn_line<R, Coef, CL>(tb + l * P, n, A.TPL, q, make_kt<Coef>(A.tau),
-                                        reinterpret_cast<const Coef *>(A.cntab), c0 + l < A.ncols);
-    else cn_line_st<R, Coef, CL>(tb + l * P, n, A.TPL, q, make_kt<Coef>(A.tau), s_tab, c0 + l < A.ncols,
-                                 A.cnd);
+    cn_line<R, Coef, CL>(tb + l * P, n, A.TPL, q, make_kt<Coef>(A.tau), reinterpret_cast<const Coef *>(A.cntab),
+                         c0 + l < A.ncols);
     __syncthreads();
     if (c0 + lc < A.ncols) {
       cx<R> *dst = A.psi + (size_t)o * A.ostride + c0 + lc;
-      // |x|^2 of the thread's CL sites summed in R (FP32: an FP64 sum per
-      // site held the FP32 final pass at the FP64 pipe's rate, 0.21 against
-      // 0.08 ms at 256^3), then accumulated in FP64 across tiles and blocks
-      R ts = (R)0;
+      double ts = 0.0;
 #pragma unroll
       for (int i = 0; i < CL; ++i) {
         const int a = r0 + i * A.TPL;
@@ -1121,7 +1102,7 @@ __global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB_CN(R)) k_cn_strided_pipe(
         dst[(size_t)a * es] = v;
         if (NORM && A.norm) ts += v.x * v.x + v.y * v.y;
       }
-      if (NORM && A.norm) acc += (double)ts;
+      if (NORM && A.norm) acc += ts;
     }
     __syncthreads();  // the buffer is refilled two iterations later
   }
