@@ -173,7 +173,7 @@ template <typename R> struct Pad { static constexpr int W = 128 / (int)sizeof(cx
 // FP32 kernels, whose register budgets (65536 / (256 x blocks)) were picked by
 // timing the 256^3 step: strided transforms 4 blocks (64 registers; 3 blocks
 // made FFT_z.U.IFFT_z 11 % slower), C2R/exponential/CN_x 3 blocks (2: 7 %
-// slower, 4: 13 % slower), pipelined CN 2 blocks (3: 14 % slower).
+// slower, 4: 13 % slower).
 #define DGPE_MAXT 256
 #ifndef DGPE_MAXT_FFT
 #define DGPE_MAXT_FFT 256  // strided transforms
@@ -1365,10 +1365,9 @@ enum { OBS_N, OBS_X2, OBS_Y2, OBS_Z2, OBS_V, OBS_N2, OBS_KX, OBS_KY, OBS_KZ, OBS
 template <typename R>
 __global__ void __launch_bounds__(256) k_obs_sites(const __grid_constant__ OArgs<R> A) {
   __shared__ double red[32];
-  constexpr int NC = 2, V = 4;  // components, sites per thread
+  constexpr int V = 4;  // sites per thread
   constexpr bool SCALED = sizeof(R) == 8;
   const int nx = A.nx, ny = A.ny, nz = A.nz;
-  const R *const psi = reinterpret_cast<const R *>(A.psi);
   const double sc = A.prm[PRM_SC];
   double acc[OBS_COUNT];
 #pragma unroll
@@ -1377,20 +1376,23 @@ __global__ void __launch_bounds__(256) k_obs_sites(const __grid_constant__ OArgs
   const unsigned g = blockIdx.x * blockDim.x + threadIdx.x, unit = g / tpr;
   const int x0 = (int)(g % tpr) * V, z = (int)(unit / chunks), ya = (int)(unit % chunks) * A.rows;
   if (z < nz) {
+    auto wide = [&](cx<R> v) {
+      return SCALED ? make_double2(sc * (double)v.x, sc * (double)v.y) : make_double2((double)v.x, (double)v.y);
+    };
     // row (zz, yy): V sites from x0, nothing beyond the grid
-    auto load = [&](int zz, int yy, double(&v)[V][NC]) {
+    auto load = [&](int zz, int yy, double2(&v)[V]) {
       if (zz >= nz || yy >= ny) {
 #pragma unroll
-        for (int i = 0; i < V * NC; ++i) v[i / NC][i % NC] = 0.0;
+        for (int i = 0; i < V; ++i) v[i] = make_double2(0.0, 0.0);
         return;
       }
-      const R *const q = psi + (((size_t)zz * ny + yy) * nx + x0) * NC;
-      R t[V * NC];
+      const cx<R> *const q = A.psi + ((size_t)zz * ny + yy) * nx + x0;
+      cx<R> t[V];
 #pragma unroll
-      for (int i = 0; i < V * NC; i += 16 / (int)sizeof(R))
+      for (int i = 0; i < V; i += 16 / (int)sizeof(cx<R>))
         *reinterpret_cast<int4 *>(t + i) = *reinterpret_cast<const int4 *>(q + i);
 #pragma unroll
-      for (int i = 0; i < V * NC; ++i) v[i / NC][i % NC] = SCALED ? sc * (double)t[i] : (double)t[i];
+      for (int i = 0; i < V; ++i) v[i] = wide(t[i]);
     };
     double X2[V];
 #pragma unroll
@@ -1399,37 +1401,30 @@ __global__ void __launch_bounds__(256) k_obs_sites(const __grid_constant__ OArgs
       X2[i] = X * X;
     }
     const double Z = A.dim == 3 ? (double)(z - nz / 2) * A.hz : 0.0;
-    double cur[V][NC], up[V][NC], far[V][NC], sz = 0.0;
+    double2 cur[V], up[V], far[V];
+    double sz = 0.0;
     load(z, ya, cur);
     const int yb = min(ny, ya + A.rows);
     for (int y = ya; y < yb; ++y) {
-      double edge[NC];
-      const size_t ie = (((size_t)z * ny + y) * nx + x0 + V) * NC;
-#pragma unroll
-      for (int c = 0; c < NC; ++c) edge[c] = x0 + V < nx ? (SCALED ? sc * (double)psi[ie + c] : (double)psi[ie + c]) : 0.0;
+      const double2 edge = x0 + V < nx ? wide(A.psi[((size_t)z * ny + y) * nx + x0 + V]) : make_double2(0.0, 0.0);
       load(z, y + 1, up);
       if (A.dim == 3) load(z + 1, y, far);
       double s = 0.0;
 #pragma unroll
       for (int i = 0; i < V; ++i) {
-        double nn = 0.0;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) nn = c ? fma(cur[i][c], cur[i][c], nn) : cur[i][c] * cur[i][c];
+        const double nn = fma(cur[i].y, cur[i].y, cur[i].x * cur[i].x);
         s += nn;
         acc[OBS_X2] = fma(X2[i], nn, acc[OBS_X2]);
         acc[OBS_N2] = fma(nn, nn, acc[OBS_N2]);
         // forward differences with zero ghosts; the (ghost, first) pair adds |psi_0|^2
         if (i == 0 && x0 == 0) acc[OBS_KX] += nn;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          const double dx = (i + 1 < V ? cur[i + 1 < V ? i + 1 : i][c] : edge[c]) - cur[i][c], dy = up[i][c] - cur[i][c];
-          acc[OBS_KX] = fma(dx, dx, acc[OBS_KX]);
-          acc[OBS_KY] = fma(dy, dy, acc[OBS_KY]);
-          if (A.dim == 3) {
-            const double dz = far[i][c] - cur[i][c];
-            acc[OBS_KZ] = fma(dz, dz, acc[OBS_KZ]);
-          }
-        }
+        auto diff = [&](double &sum, double2 next) {
+          const double2 d = next - cur[i];
+          sum = fma(d.y, d.y, fma(d.x, d.x, sum));
+        };
+        diff(acc[OBS_KX], i + 1 < V ? cur[i + 1 < V ? i + 1 : i] : edge);
+        diff(acc[OBS_KY], up[i]);
+        if (A.dim == 3) diff(acc[OBS_KZ], far[i]);
       }
       if (!isfinite(s)) acc[OBS_BAD] += 1.0;
       const double Y = (double)(y - ny / 2) * A.hy;
@@ -1437,7 +1432,7 @@ __global__ void __launch_bounds__(256) k_obs_sites(const __grid_constant__ OArgs
       if (y == 0) acc[OBS_KY] += s;
       sz += s;
 #pragma unroll
-      for (int i = 0; i < V * NC; ++i) cur[i / NC][i % NC] = up[i / NC][i % NC];
+      for (int i = 0; i < V; ++i) cur[i] = up[i];
     }
     acc[OBS_N] = sz;
     acc[OBS_Z2] = Z * Z * sz;
