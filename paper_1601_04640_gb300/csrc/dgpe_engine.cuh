@@ -1451,18 +1451,37 @@ template <typename R> struct EngineT : Engine {
       case 4: return 16;    // 8 complex additions
       case 5: return 48;
       case 8: return 60;    // two radix-4 (32) + two w8 rotations (12) + 8 additions (16)
+      case 12: return 112;  // four of 3 points, three of 4 (no twiddles)
+      case 20: return 272;  // five of 4 points, four of 5
       case 16: return 176;  // eight radix-4 (128) + eight inner twiddle rotations (48)
       default: return 0;
     }
   }
-  static double fft_line_flops(const FftPlan &pl) {
+  // A line of n points whose stage at sub-transform length n / left has radix
+  // next(left).
+  template <class F> static double stages_flops(int n, F next) {
     double f = 0.0;
-    for (int s = 0; s < pl.ns; ++s) {
-      const double nb = (double)pl.n / pl.rad[s];
-      f += nb * codelet_flops(pl.rad[s]);
-      if (s > 0) f += nb * (pl.rad[s] - 1) * 6.0;
+    for (int left = n; left > 1;) {
+      const int r = next(left);
+      f += (double)n / r * (codelet_flops(r) + (left < n ? 6.0 * (r - 1) : 0.0));
+      left /= r;
     }
     return f;
+  }
+  double fft_line_flops(int axis) const {
+    const FftPlan &pl = axis == 0 ? plx : axis == 1 ? ply : plz;
+    const int n = axis == 0 ? nx : axis == 1 ? ny : nz;
+    if (fine) return stages_flops(n, [](int left) { return fine_radix(left); });
+    if (sizeof(R) == 4 && (axis > 0 || rows_back)) {  // the first radix, then as in row_radix, ct_radix_cols
+      const int ept = variant_ept_s(var[axis], EPT_S), first = axis > 0 && ept == 16 ? 0 : ept;
+      return stages_flops(n, [&](int left) {
+        if (left == n && first && n % first == 0) return first;
+        return axis == 0 ? (ept == 16 && left % 16 == 0 ? 16 : ept == 16 && left % 8 == 0 ? 8 : left % 4 == 0 ? 4 : 2)
+                         : ct_radix(left, ept, 0);
+      });
+    }
+    int s = 0;
+    return stages_flops(n, [&](int) { return pl.rad[s++]; });
   }
   // exponential substep per site.  FP32 and imaginary time: V (1), scaled
   // psi (2), density (3), theta (5 with the dipolar term, else 3), the factor
@@ -1478,16 +1497,28 @@ template <typename R> struct EngineT : Engine {
     if (imag) return 1 + 2 + 3 + th + 1 + 4;
     return 1 + 2 + 3 + th + 11.0 + 8;
   }
-  // Thomas solve per site: line-serial (forward right-hand side, forward
-  // elimination, back substitution) or chunk-parallel (chunk passes, the two
-  // lane scans amortised over the chunk, fix-ups)
+  // Crank-Nicolson solve per site: line-serial (forward right-hand side, forward
+  // elimination, back substitution), chunks with constant coefficients
+  // (difference, two recurrences, three fix-ups of the first J sites, the last
+  // product; FP64 small grids: fix-ups of every site), or chunks with tables
+  // (chunk passes, the two lane scans amortised over the chunk, fix-ups)
   double cn_flops_per_site(int axis) const {
     if (cn_serial) return imag ? 16.0 : 28.0;
     // a real state: one complex solve with real coefficients advances two sites
-    if (rpsi) return 0.5 * cn_flops_chunked(axis);
-    return cn_flops_chunked(axis);
+    return (rpsi ? 0.5 : 1.0) * cn_flops_chunked(axis);
   }
   double cn_flops_chunked(int axis) const {
+    const double m = imag ? 4.0 : 8.0;  // a multiply-add of a complex number
+    if (fine) {
+      const int cl = fine_chunk(axis == 0 ? nx : axis == 1 ? ny : nz), tpl = (axis == 0 ? nx : axis == 1 ? ny : nz) / cl;
+      const int dl = imag ? fine_kr[axis].dl : fine_kc[axis].dl, nE = imag ? fine_kr[axis].nE : fine_kc[axis].nE;
+      return 6.0 + 5.0 * m + m * nE / tpl + 2.0 * m * (dl ? dl : std::log2((double)tpl)) / cl;
+    }
+    const int dl = imag ? cn_kr[axis].dl : cn_kc[axis].dl, J = imag ? cn_kr[axis].J : cn_kc[axis].J;
+    if (dl && (axis > 0 || rows_back)) {
+      const int cl = axis == 0 ? rows_chunk(nx) : cn[axis].C;
+      return 6.0 + 3.0 * m + (3.0 * J + 2.0 * dl) * m / cl;
+    }
     const int cl = (axis == 0) ? x_C : cn[axis].C;
     const int tpl = (axis == 0) ? x_TPL : cn[axis].TPL;
     const double lg = std::log2((double)std::max(tpl, 1));
@@ -1500,12 +1531,12 @@ template <typename R> struct EngineT : Engine {
     const double N = (double)nsites, pairs = (double)((nrows + 1) / 2);
     const double norm = (imag ? 4.0 : 0.0);  // FP64 |x|^2 accumulation of the final pass
     switch (v[i]) {
-      case PS_DENS_R2C: return (rpsi ? 2.0 : 4.0) * N + pairs * fft_line_flops(plx) + pairs * (nx / 2 + 1) * 8.0;
-      case PS_FFT_Y: case PS_IFFT_Y: return (double)ncol_spec * nz * fft_line_flops(ply);
-      case PS_FFT_Z_U: return (double)ncol_spec * ny * (2.0 * fft_line_flops(plz) + 2.0 * nz);
-      case PS_FFT_Y_U: return (double)ncol_spec * (2.0 * fft_line_flops(ply) + 2.0 * ny);
+      case PS_DENS_R2C: return (rpsi ? 2.0 : 4.0) * N + pairs * fft_line_flops(0) + pairs * (nx / 2 + 1) * 8.0;
+      case PS_FFT_Y: case PS_IFFT_Y: return (double)ncol_spec * nz * fft_line_flops(1);
+      case PS_FFT_Z_U: return (double)ncol_spec * ny * (2.0 * fft_line_flops(2) + 2.0 * nz);
+      case PS_FFT_Y_U: return (double)ncol_spec * (2.0 * fft_line_flops(1) + 2.0 * ny);
       case PS_P1: case PS_P1_NOCN: {
-        double f = (has_dip ? pairs * fft_line_flops(plx) : 0.0) + N * exp_flops_per_site();
+        double f = (has_dip ? pairs * fft_line_flops(0) : 0.0) + N * exp_flops_per_site();
         if (v[i] == PS_P1) f += N * cn_flops_per_site(0);
         return f;
       }

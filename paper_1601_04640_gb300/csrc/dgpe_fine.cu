@@ -25,7 +25,6 @@ constexpr int fine_cl(int n) {
   while (n / cl > 32) cl *= 2;
   return cl;
 }
-constexpr int fine_radix(int left) { return left % 4 == 0 ? 4 : left % 5 == 0 ? 5 : left % 3 == 0 ? 3 : 2; }
 
 // Stockham stages over NL lines of a tile in shared memory, T threads.  Lines
 // along the threads (COLS: element a of line l at a NL + l, NL = 2^ll) or one

@@ -33,6 +33,8 @@ struct FineArgs {
   long long es, os;
   int has_dip, final_pass, norm, nsm, early;
 };
+// radix of a transform's stage with `left` points to go
+constexpr int fine_radix(int left) { return left % 4 == 0 ? 4 : left % 5 == 0 ? 5 : left % 3 == 0 ? 3 : 2; }
 // points per lane of the solve (n / that is a power of two <= 32)
 int fine_chunk(int n);
 // density (src 0: sc^2 |psi|^2, 1: dens_in, 2: of a real state) + R2C along x
