@@ -85,9 +85,15 @@ extern "C" {
 #define DGPE_FLAG_NO_GRAPH 1u   /* launch the passes directly instead of
                                    replaying a captured CUDA graph */
 #define DGPE_FLAG_CN_SERIAL 2u  /* FP64 form: solve every CN line serially,
-                                   one thread per line (the default once the
-                                   grid has >= 8192 lines per axis); the FP32
-                                   form returns DGPE_EUNSUPPORTED */
+                                   one thread per line.  The default once the
+                                   grid has >= 8192 lines per axis, except on
+                                   grids that take the small-grid passes (up to
+                                   2^20 sites; 2^19 where all three sides are
+                                   powers of two up to 128; 2^23 where nx is
+                                   5 2^k): there only in real time without
+                                   dipoles.  The flag also keeps a grid from
+                                   the small-grid passes.  The FP32 form returns
+                                   DGPE_EUNSUPPORTED */
 #define DGPE_FLAG_CN_CHUNKED 4u /* FP64 form: always use the chunk-parallel
                                    CN solve (exclusive with CN_SERIAL) */
 #define DGPE_FLAG_STRANG 8u     /* real time: second-order (Strang) splitting,
@@ -116,13 +122,19 @@ extern "C" {
 #define DGPE_FLAG_P1_ONESHOT 32u /* FP32 bulk: run the two x-line passes
                                    (density + R2C; C2R, exponential, CN_x) as
                                    one CTA per tile instead of the default
-                                   persistent CTAs fed by bulk asynchronous
+                                   persistent warps fed by bulk asynchronous
                                    copies, and the strided transforms as
-                                   register-fed tiles instead of persistent
-                                   CTAs fed by tensor-map copies (same
-                                   arithmetic, except that the 3D z-pass
-                                   then reads U(k) from its FP32 table
-                                   instead of evaluating it in FP32) */
+                                   register-fed tiles of up to 16 columns
+                                   instead of persistent CTAs fed by tensor-map
+                                   copies (3D) or narrow tiles (2D).  The two
+                                   agree to FP32 rounding, some 1e-7 of the
+                                   state per step, not to the last bit: CN_x
+                                   then runs from LU tables with chunk scans
+                                   instead of constant coefficients with an
+                                   inflow cut at 2^-32, exponents above 1/8 call
+                                   the library instead of a longer series, and
+                                   the 3D z-pass reads U(k) from its FP32 table
+                                   instead of evaluating it in FP32 */
 
 #define DGPE_FLAG_BATCH_CLASSES 64u /* batched form (set on any problem): step
                                    the batch as per-size-class batched kernels
@@ -229,10 +241,10 @@ const char *dgpe_pass_name(dgpe_t h, int i);
 double dgpe_pass_bytes(dgpe_t h, int i);
 
 /* Floating-point operations of pass i per launch, an FMA counting 2: the
- * operation count of the pass's algorithm (FFT codelets and twiddles, pair
- * packing of the real transforms, the exponential substep with sin and
- * cos - 1 by Taylor series (expm1 counted as one operation), the Thomas
- * recurrences).  0 for an index out of range or a NULL handle. */
+ * operation count of the form of the pass that runs (FFT codelets and twiddles,
+ * pair packing of the real transforms, the exponential substep with sin and
+ * cos - 1 by Taylor series (expm1 counted as one operation), the
+ * Crank-Nicolson recurrences).  0 for an index out of range or a NULL handle. */
 double dgpe_pass_flops(dgpe_t h, int i);
 
 /* Kernels this handle has launched since it was created (each replay of the

@@ -282,7 +282,8 @@ template <typename R> struct EngineT : Engine {
   unsigned *counter = nullptr;
   FftPlan plx{}, ply{}, plz{}, plx_s{};
   double tau[3] = {0, 0, 0};
-  // chunk-scan reach of the FP32 chunk-parallel CN solve per axis (cn_line_st)
+  // chunk-scan reach of the table forms of the chunk-parallel CN solve per axis
+  // (cn_line, cn_line_st, the table form of k_cn_cols)
   int cn_dlim[3] = {0, 0, 0};
   // constant-coefficient CN form of each axis (FP32 bulk; dl = 0: tables):
   // imaginary time, real time, and real time conjugated for the reverse step

@@ -548,7 +548,8 @@ __global__ void __launch_bounds__(DGPE_MAXT, DGPE_MINB_P1(R)) k_c2r_x_exp_cnx_ba
 
 // ----------------------------------------------- P1, FP32 pipelined form
 // The x-line pass of the FP32 bulk (complex state, power-of-two nx) as a
-// persistent pipeline.  A tile is the 2 LP consecutive rows of psi and of the
+// persistent pipeline, for coefficients that decay too slowly for the constant
+// form of the row passes (dgpe_rows_back.cuh).  A tile is the 2 LP consecutive rows of psi and of the
 // half spectrum that the one-shot kernel above gives a CTA; both are
 // contiguous blocks, so one thread brings them into shared memory with two
 // bulk copies that complete on an mbarrier (no per-element load

@@ -1,7 +1,7 @@
 // dgpe_lines.h -- arguments and launchers of the register-resident line
 // passes of the FP32 bulk (dgpe_rows*.cu: x-rows; dgpe_cols.cu: the strided
 // Crank-Nicolson solves along y and z).  Each kernel is compiled once, in
-// those units; the solver and the batched form call the launchers.
+// those units; the solver (and dgpe_noalloc.cu, the row passes) calls the launchers.
 #pragma once
 
 #include <cuda.h>  // CUtensorMap
