@@ -1,16 +1,17 @@
-// dgpe_fine.cu -- the passes of one step in FP64 on grids of up to some 10^5
+// dgpe_fine.cu -- the passes of one step in FP64 on grids of up to some 10^6
 // sites (the paper's calcpsidd2, calcnu, calclux/y/z, calcnorm).
 //
-// Such a grid has fewer warps than the GPU has schedulers, so a pass takes what
-// one warp executes: every instruction of a lone warp costs some 10 cycles, an
-// FP64 one 64 (2 FMA per SM and clock), and code that runs once is fetched as
+// The smaller ones have fewer warps than the GPU has schedulers, so a pass takes
+// what one warp executes: every instruction of a lone warp costs some 10 cycles,
+// an FP64 one 64 (2 FMA per SM and clock), and code that runs once is fetched as
 // it runs.  So a thread holds few points (one radix-4 or -5 butterfly, chunks of
 // 3 to 5 points of a line), lengths are compile-time constants, the state goes
 // from global memory to registers and back, and the solve needs no tables.
 // A step of 32^3 in imaginary time went from 123 to 43 us, of a 96 x 160 plane
-// from 156 to 38, of 256^2 from 129 to 57 and of 64 x 80 x 64 from 197 to 141;
-// what is left is some 6 us per pass: launch, a cold start and one warp's chain
-// of FP64 instructions.
+// from 156 to 37, of 256^2 from 129 to 56, of 64^3 from 143 to 118 (real time 183
+// to 143) and of 64 x 80 x 64 in real time from 250 to 174; what is left on the
+// smallest is some 6 us per pass: launch, a cold start and one warp's chain of
+// FP64 instructions.
 #include <algorithm>
 
 #include "dgpe_kernels.cuh"
