@@ -150,11 +150,13 @@ __device__ __forceinline__ void fine_solve(double2 (&v)[CL], int q, const FineCn
   double2 acc = make_double2(0.0, 0.0);
 #pragma unroll
   for (int i = 0; i < CL; ++i) {
-    // (2 psi_a - psi_{a-1}) - psi_{a+1} in this order: where psi is smooth both differences are exact, while a
+    // (2 psi_a - psi_{a-1}) - psi_{a+1}, one after the other: where psi is smooth both differences are exact, while a
     // rounded psi_{a-1} + psi_{a+1} leaves 2^-53 psi, which -2 kt m and the two recurrences amplify (two solves of
     // 32 to 256 points at kt between 1 and 10, relative L2: 1.9e-16 instead of 5.2e-16 in real time)
-    const double2 l = i ? v[i - 1] : prev, r = i + 1 < CL ? v[i + 1 < CL ? i + 1 : i] : next;
-    acc = coef_fma(K.al, acc, make_double2(fma(2.0, v[i].x, -l.x) - r.x, fma(2.0, v[i].y, -l.y) - r.y));
+    // psi_{a+1} first at the chunk's first point, whose psi_{a-1} comes by a shuffle (96 x 160: 2014 -> 1999 us for
+    // 50 steps and the observables).
+    const double2 l = i ? v[i - 1] : prev, r = i + 1 < CL ? v[i + 1 < CL ? i + 1 : i] : next, f = i ? l : r, g = i ? r : l;
+    acc = coef_fma(K.al, acc, make_double2(fma(2.0, v[i].x, -f.x) - g.x, fma(2.0, v[i].y, -f.y) - g.y));
     y[i] = acc;
   }
   double2 in = make_double2(0.0, 0.0);
